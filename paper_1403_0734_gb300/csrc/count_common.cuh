@@ -311,6 +311,15 @@ __device__ __forceinline__ void build_rows(const Ctx& c, const int32_t* sL, cons
     }
 }
 
+// Row widths (words) the closing kernels (close.cu) are built for: 1..6, 8,
+// 12, 16; the number of the narrowest one that holds a set of n elements.
+constexpr int kCloseBins = 9;
+__host__ __device__ __forceinline__ int close_bin(int n)
+{
+    const int w = (n + 31) >> 5;
+    return w <= 6 ? w - 1 : (w <= 8 ? 6 : (w <= 12 ? 7 : 8));
+}
+
 // Opt a kernel in to `smem` bytes of dynamic shared memory.  The default
 // limit (48 KB) covers static and dynamic shared memory together, so the
 // attribute is set whenever the dynamic part alone comes near it.

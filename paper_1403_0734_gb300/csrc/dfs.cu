@@ -31,6 +31,9 @@
 namespace kc {
 
 int num_sms();
+bool close_supported(int W, int k, int64_t items);
+kc_status close_launch(const cc::Ctx& c, int W, int dmax, uint32_t* tiles, int64_t tile_words, int RS, unsigned int* ctr,
+                       cudaStream_t s);
 
 namespace {
 
@@ -40,6 +43,7 @@ using cc::mask_above;
 using cc::mask_below;
 using cc::warp_sum64;
 
+constexpr int kCloseCursors = 48;  // counters of close_launch, in the task counters' place
 constexpr int kMaxLev = 5;  // register stack levels: k - 3 <= 5, i.e. k <= 8
 
 }  // namespace
@@ -1082,9 +1086,11 @@ __global__ void __launch_bounds__(256, 4) k_dfs_reg(Ctx cb, int W, int R, int cl
 }
 
 // G+(u) of every owner of the class, built once into its global tile (the
-// shared-memory row layout, d rows of RS words), for the split search.
+// shared-memory row layout, d rows of RS words), for the split search and the
+// closing kernels.
 template <bool PV, bool COL, int WM>
-__global__ void __launch_bounds__(256) k_tile_build(Ctx cb, int W, uint32_t* tiles, int64_t tile_words)
+__global__ void __launch_bounds__(256) k_tile_build(Ctx cb, int W, uint32_t* tiles, int64_t tile_words,
+                                                    unsigned int* sizes)
 {
     extern __shared__ __align__(16) uint32_t smem[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, NW = blockDim.x >> 5;
@@ -1094,6 +1100,7 @@ __global__ void __launch_bounds__(256) k_tile_build(Ctx cb, int W, uint32_t* til
     uint32_t* sCol = smem + lay.col;
     uint32_t* sA = smem + lay.A;
     __shared__ long long s_item;
+    __shared__ unsigned int s_bins[cc::kCloseBins];
     for (;;) {
         if (threadIdx.x == 0) s_item = (long long)atomicAdd(cb.cursor, 1ull);
         __syncthreads();
@@ -1116,6 +1123,23 @@ __global__ void __launch_bounds__(256) k_tile_build(Ctx cb, int W, uint32_t* til
         cc::span_table_build(T, sL, d, kSpanWords);
         cc::build_rows<PV, COL>(c, sL, sCol, d, sA, RS, wid, NW, lane, ur, &T);
         __syncthreads();
+        if (PV && WM > 0 && sizes) {
+            // for the closing kernels: the size of every row's candidate set (the
+            // elements above it) in the row's first spare word, and their number
+            // by row width
+            if (threadIdx.x < cc::kCloseBins) s_bins[threadIdx.x] = 0u;
+            __syncthreads();
+            for (int e = threadIdx.x; e < d; e += blockDim.x) {
+                uint32_t* Ae = sA + (int64_t)e * RS;
+                int n = __popc(Ae[e >> 5] & mask_above(e & 31));
+                for (int w = (e >> 5) + 1; w < WM; ++w) n += __popc(Ae[w]);
+                Ae[WM] = (uint32_t)n;
+                if (n >= 4) atomicAdd(&s_bins[cc::close_bin(n)], 1u);
+            }
+            __syncthreads();
+            if (threadIdx.x < cc::kCloseBins && s_bins[threadIdx.x])
+                atomicAdd(&sizes[threadIdx.x], s_bins[threadIdx.x]);
+        }
         uint4* dst = (uint4*)(tiles + oi * tile_words);
         const uint4* src = (const uint4*)sA;
         for (int64_t j = threadIdx.x; j < ((int64_t)d * RS + 3) / 4; j += blockDim.x) dst[j] = src[j];
@@ -1159,14 +1183,14 @@ int64_t dfs_tile_words(int W, int k, int64_t items, int parts)
     if ((parts > 0 ? parts : parts_per_owner(W, k)) <= 1 || items <= 0) return 0;
     const int WM = W <= 16 ? W : 0;
     const int64_t per = 32LL * W * row_stride(W, WM);
-    return per * items + (items + 3);  // tiles, then the task counters
+    return per * items + (items + kCloseCursors + 3);  // tiles, then the task counters
 }
 
 // Launch the shared-memory class of width W (words) over its queue range.
 // With an allocator and R > 1 the owners' rows are built once into global
 // tiles (k_tile_build) and the R parts copy them; without one (the
 // allocation-free entry point) every owner is searched by one CTA.
-kc_status dfs_reg_launch(const cc::Ctx& c, int W, bool pv, bool col, Scratch* sc, int parts, cudaStream_t s)
+kc_status dfs_reg_launch(const cc::Ctx& c, int W, int dmax, bool pv, bool col, Scratch* sc, int parts, cudaStream_t s)
 {
     const int sms = num_sms();
     int R = parts > 0 ? parts : parts_per_owner(W, c.k);
@@ -1187,18 +1211,29 @@ kc_status dfs_reg_launch(const cc::Ctx& c, int W, bool pv, bool col, Scratch* sc
     if (R > 1) {
         KC_TRY(sc->get(&tiles, dfs_tile_words(W, c.k, c.nitems, R)));
         ctr = tiles + tile_words * c.nitems;
-        KC_CK(cudaMemsetAsync(ctr, 0, (size_t)c.nitems * sizeof(unsigned int), s));
+        KC_CK(cudaMemsetAsync(ctr, 0, (size_t)(c.nitems + kCloseCursors) * sizeof(unsigned int), s));
+    }
+    // one pass over the owners of the class that writes their tiles
+    auto build_tiles = [&](auto build, unsigned int* sizes) -> kc_status {
+        const RLayout bl = make_rlayout(W, RS, false, col, 8);
+        const size_t bsm = (size_t)bl.total * 4;
+        KC_CK(cc::allow_smem(build, bsm));
+        const int bgrid = (int)std::min<int64_t>(c.nitems, (int64_t)sms * cc::blocks_per_sm(build, 256, bsm));
+        build<<<bgrid, 256, bsm, s>>>(c, W, tiles, tile_words, sizes);
+        KC_LAUNCHED();
+        return KC_OK;
+    };
+    if (R > 1 && g_complement && close_supported(W, c.k, c.nitems)) {
+        // tiles with the candidate-set sizes, then the sets of every size (close.cu)
+        if (col) KC_TRY(W == 16 ? build_tiles(k_tile_build<true, true, 16>, ctr) : build_tiles(k_tile_build<true, true, 8>, ctr));
+        else KC_TRY(W == 16 ? build_tiles(k_tile_build<true, false, 16>, ctr) : build_tiles(k_tile_build<true, false, 8>, ctr));
+        return close_launch(c, W, dmax, tiles, tile_words, RS, ctr, s);
     }
     auto pick = [&](auto kern, auto build) -> kc_status {
         if (R > 1) {
             // the build pass takes owners from the class cursor; the search
             // pass then counts items from a second cursor (the slot's next word)
-            const RLayout bl = make_rlayout(W, RS, false, col, 8);
-            const size_t bsm = (size_t)bl.total * 4;
-            KC_CK(cc::allow_smem(build, bsm));
-            const int bgrid = (int)std::min<int64_t>(c.nitems, (int64_t)sms * cc::blocks_per_sm(build, 256, bsm));
-            build<<<bgrid, 256, bsm, s>>>(c, W, tiles, tile_words);
-            KC_LAUNCHED();
+            KC_TRY(build_tiles(build, nullptr));
         }
         cc::Ctx cs = c;
         if (R > 1) cs.cursor = c.cursor + kc::kOwnerSlots;  // a fresh zeroed cursor for the search
