@@ -119,7 +119,9 @@ typedef struct {
     int64_t m;              /* undirected edges = sum over u of |Gamma+(u)| */
     int32_t max_dplus;      /* max |Gamma+(u)|, at most 2 sqrt(m) (App. B, Thm I) */
     int64_t wedges;         /* sum over u of C(|Gamma+(u)|, 2): Map 2 pairs (App. B, Thm 1) */
-    int64_t device_bytes;   /* device memory held by the handle */
+    int64_t device_bytes;   /* device memory held by the handle: lists, offsets, per-vertex
+                               arrays, and an adjacency bitmap of the last ranks of the order
+                               (at most 16384 of them, and about 4 m bytes) */
 } kc_graph_info;
 
 /* Statistics of an oriented graph (host struct).  Errors: KC_EINVAL. */
@@ -323,9 +325,10 @@ kc_status kc_count_batch(const kc_graph* const* gs, int ng, int k, unsigned flag
  *   KC_PARAM_COMPACT_LO, KC_PARAM_COMPACT_HI  candidate sets of the ordered
  *       search with LO..HI elements (HI <= 64, default 1..64; HI = 0 off) are
  *       finished on a compact register copy of their induced subgraph.
- *   KC_PARAM_TRI  1 (default): exact k = 3 counts take the triangle path --
- *       each y of Gamma+(x_i) found in Gamma+(u) is counted directly (node
- *       iterator, no G+(u) bitmap); 0: the bitmap path used for larger k.
+ *   KC_PARAM_TRI  1 (default): exact k = 3 counts of owners with more than 64
+ *       elements take the triangle path -- each y of Gamma+(x_i) found in
+ *       Gamma+(u) is counted directly (node iterator, no G+(u) bitmap); 0: the
+ *       bitmap path used for larger k.
  *   KC_PARAM_COMPLEMENT  1 (default): the ordered search of the 4-, 8- and
  *       16-word classes closes a candidate set C that still needs three
  *       vertices through the complement of G[C] when C is dense (non-edges

@@ -403,7 +403,7 @@ kc_status kc_count_batch(const kc_graph* const* gs, int ng, int k, unsigned flag
     int Wh = 1;
     int64_t nheavy = 0;
     for (int i = 0; i < ng; ++i) {
-        hd[(size_t)i] = {gs[i]->offp, gs[i]->adjp, gs[i]->queue, gs[i]->perm};
+        hd[(size_t)i] = kc::cc::desc_of(gs[i]);
         Wh = std::max(Wh, (gs[i]->max_dplus + 31) / 32);
         int64_t q0 = 0, q1 = 0;
         kc::class_range(gs[i], k, 0, &q0, &q1);
@@ -492,7 +492,7 @@ kc_status kc_batch_create(const kc_graph* const* gs, int ng, int k, unsigned fla
     int Wh = 1;
     int64_t nheavy = 0;
     for (int i = 0; i < ng; ++i) {
-        hd[(size_t)i] = {gs[i]->offp, gs[i]->adjp, gs[i]->queue, gs[i]->perm};
+        hd[(size_t)i] = kc::cc::desc_of(gs[i]);
         Wh = std::max(Wh, (gs[i]->max_dplus + 31) / 32);
         int64_t q0 = 0, q1 = 0;
         kc::class_range(gs[i], k, 0, &q0, &q1);

@@ -76,6 +76,7 @@ __global__ void __launch_bounds__(256) k_close_list(Ctx cb, Lists L, int chunks,
     }
 }
 
+// Sets a team takes per cursor step at most (1 for teams of several warps).
 constexpr int sets_taken(int WC) { return WC == 1 ? 8 : (WC == 2 ? 4 : 1); }
 
 // The sets of one width: a team takes list entries from the cursor (several
@@ -84,9 +85,9 @@ constexpr int sets_taken(int WC) { return WC == 1 ? 8 : (WC == 2 ? 4 : 1); }
 // each set, and closes it.  Memberships go to global memory at once (a few per
 // cent of a set's work, and it leaves the shared memory to the sets).
 template <int WC, int NEED>
-__global__ void __launch_bounds__(cta_threads(WC), ctas_per_sm(WC)) k_close(Ctx cb, Lists L, int bin, unsigned int* cursor)
+__global__ void __launch_bounds__(cta_threads(WC), ctas_per_sm(WC)) k_close(Ctx cb, Lists L, int bin, int take, unsigned int* cursor)
 {
-    constexpr int NT = team_threads(WC), NW = NT / 32, kTake = sets_taken(WC);
+    constexpr int NT = team_threads(WC), NW = NT / 32;
     constexpr TeamLayout l = team_layout(WC, 16, NW);
     extern __shared__ __align__(16) char smem_close[];
     __shared__ unsigned int s_item;
@@ -102,7 +103,7 @@ __global__ void __launch_bounds__(cta_threads(WC), ctas_per_sm(WC)) k_close(Ctx 
     for (;;) {
         unsigned int item = 0;
         if (NT == 32) {
-            if (lane == 0) item = atomicAdd(cursor, (unsigned)kTake);
+            if (lane == 0) item = atomicAdd(cursor, (unsigned)take);
             item = __shfl_sync(kFull, item, 0);
         } else {
             if (threadIdx.x == 0) s_item = atomicAdd(cursor, 1u);
@@ -111,14 +112,14 @@ __global__ void __launch_bounds__(cta_threads(WC), ctas_per_sm(WC)) k_close(Ctx 
             __syncthreads();
         }
         if (item >= sets) break;
-        const int have = (int)min((unsigned)kTake, sets - item);
+        const int have = (int)min((unsigned)take, sets - item);
         uint32_t ent = 0;
-        int32_t own = 0;
         int64_t at = 0;
         int deg = 0, size = 0;
         if (lane < have) {
             ent = L.entry(first + item + (unsigned)lane);
             Ctx cl;
+            int32_t own;
             cc::resolve(cb, ent >> 10, cl, own);
             at = cl.offp[own];
             deg = (int)(cl.offp[own + 1] - at);
@@ -127,11 +128,11 @@ __global__ void __launch_bounds__(cta_threads(WC), ctas_per_sm(WC)) k_close(Ctx 
 #pragma unroll 1
         for (int i = 0; i < have; ++i) {
             const uint32_t e = __shfl_sync(kFull, ent, i);
-            int32_t r = __shfl_sync(kFull, own, i);
             const int64_t b = __shfl_sync(kFull, at, i);
             const int Wd = (__shfl_sync(kFull, deg, i) + 31) >> 5, n = __shfl_sync(kFull, size, i), e1 = (int)(e & 1023u);
-            Ctx c = cb;
-            if (cb.ng) cc::resolve(cb, e >> 10, c, r);  // (the graph's pointers)
+            Ctx c;
+            int32_t r;
+            cc::resolve(cb, e >> 10, c, r);  // (always an item)
             const uint32_t* __restrict__ T = L.tiles + (int64_t)(e >> 10) * L.tile_words;
             list_set<WC, NT>(t, upper_word(T, L.RS, e1, Wd, lane), Wd, lane, wid);
             sync<NT>();
@@ -171,8 +172,10 @@ kc_status launch_bin(const Ctx& c, const Lists& L, int bin, unsigned int* cursor
     auto kern = k_close<WC, NEED>;
     KC_CK(cc::allow_smem(kern, smem));
     const int64_t room = (int64_t)num_sms() * cc::blocks_per_sm(kern, cta_threads(WC), smem);
+    // sets per cursor step: one for classes too small to give every team several
     const int grid = (int)std::min<int64_t>((c.nitems * L.rows + teams - 1) / teams, room);
-    kern<<<grid, cta_threads(WC), smem, s>>>(c, L, bin, cursor);
+    const int take = c.nitems * L.rows > 64 * room * teams ? sets_taken(WC) : 1;
+    kern<<<grid, cta_threads(WC), smem, s>>>(c, L, bin, take, cursor);
     KC_LAUNCHED();
     return KC_OK;
 }

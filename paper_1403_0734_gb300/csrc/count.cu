@@ -92,28 +92,34 @@ __device__ __forceinline__ unsigned long long leaf2_w1(uint32_t C, uint32_t up, 
     return (unsigned long long)__reduce_add_sync(kFull, e);
 }
 
+constexpr int kW1Take = 8;  // owners a warp takes per cursor step at most
+
 template <bool PV, bool COL>
-__global__ void __launch_bounds__(256) k_count_w1(Ctx cb)
+__global__ void __launch_bounds__(256) k_count_w1(Ctx cb, int take)
 {
+    __shared__ cc::SmallBuf<1> s_buf[8];
     const int lane = threadIdx.x & 31;
+    cc::SmallBuf<1>& sb = s_buf[threadIdx.x >> 5];
     const int r0 = cb.k - 1;  // vertices to choose inside G+(u)
-    for (;;) {
-        unsigned long long pos = 0;
-        if (lane == 0) pos = atomicAdd(cb.cursor, 1ull);
-        pos = __shfl_sync(kFull, pos, 0);
+    cc::TotalSum total(cb.total);
+    cc::Owners own(take);
+    while (own.next(cb, lane)) {
         Ctx c;
         int32_t r;
-        if (!cc::resolve(cb, (int64_t)pos, c, r)) break;
-        const int64_t b = c.offp[r];
-        const int d = (int)(c.offp[r + 1] - b);
-        const int32_t x = lane < d ? c.adjp[b + lane] : INT_MAX;
-        uint32_t col = 0;
+        int64_t b;
+        int d;
+        own.take(cb, lane, c, r, b, d);
+        int32_t xs[1] = {lane < d ? c.adjp[b + lane] : INT_MAX};
+        const int32_t x = xs[0];
+        uint32_t cols[1] = {0u};
         const int32_t ur = COL ? c.perm[r] : 0;
-        if (COL && lane < d) col = cc::sample_label(c, ur, c.perm[x]);
-        if (COL) col = cc::class_flag_w1(c, col, d, r0, lane);
+        if (COL && lane < d) cols[0] = cc::sample_label(c, ur, c.perm[x]);
+        if (COL) cols[0] = cc::class_flag_w1(c, cols[0], d, r0, lane);
 
-        // (b) rows: lane j searches x_j in each 32-entry chunk of Gamma+(x_i)
-        const uint32_t up = cc::build_rows_w1<COL>(c, x, d, col, ur, lane);
+        // (b) rows
+        uint32_t rows[1][1];
+        cc::build_rows_small<1, COL>(c, xs, d, cols, ur, sb, lane, rows);
+        const uint32_t up = rows[0][0];
         const uint32_t A = PV ? (up | cc::lower_rows_w1(up, d, lane)) : up;
 
         // (c) depth-first search; level t's state of the chain is kept in lane t
@@ -165,14 +171,15 @@ __global__ void __launch_bounds__(256) k_count_w1(Ctx cb)
                 }
             }
         }
+        total.add(c.total, tot, lane);
         if (lane == 0) {
-            add_total(c.total, tot);
             if (c.po) c.po[r] = tot;
             if (PV && tot) atomicAdd(&c.pv[r], tot);
             if (cw && wk) atomicAdd(c.work, wk);
         }
         if (PV && lane < d && pvl) atomicAdd(&c.pv[x], pvl);
     }
+    total.flush(lane);
 }
 
 // ----------------------------------------------------- wide classes (CTA)
@@ -469,8 +476,8 @@ kc_status launch_slot_dfs(int slot, int Wh, const Ctx& c, uint32_t* heavy, int64
     }
     if (slot == kOwnerSlots - 1) {
         auto kern = k_count_w1<PV, COL>;
-        const int grid = (int)std::min<int64_t>((c.nitems + 7) / 8, (int64_t)sms * cc::blocks_per_sm(kern, 256, 0));
-        kern<<<grid, 256, 0, s>>>(c);
+        const cc::OwnerSteps st = cc::owner_steps(c.nitems, 8, (int64_t)sms * cc::blocks_per_sm(kern, 256, 0), kW1Take);
+        kern<<<st.grid, 256, 0, s>>>(c, st.take);
         KC_LAUNCHED();
         return KC_OK;
     }
@@ -492,7 +499,12 @@ kc_status launch_slot_dfs(int slot, int Wh, const Ctx& c, uint32_t* heavy, int64
 kc_status launch_slot(int slot, int Wh, const Ctx& c, bool pv, bool col, uint32_t* heavy, int64_t heavy_words,
                       Scratch* sc, const Plan* plan, cudaStream_t s)
 {
-    if (c.k == 3 && !col && tri_enabled()) return tri_launch_slot(slot, Wh, c, pv, s);  // no bitmaps for k = 3
+    if (c.k == 3 && !col && tri_enabled()) {  // no bitmaps for k = 3 but in registers
+        if (slot_words(slot) == 1 || slot_words(slot) == 2)
+            return pv ? launch_slot_dfs<true, false>(slot, Wh, c, heavy, heavy_words, sc, 1, s)
+                      : launch_slot_dfs<false, false>(slot, Wh, c, heavy, heavy_words, sc, 1, s);
+        return tri_launch_slot(slot, Wh, c, pv, s);
+    }
     const int algo = plan ? plan->algo[slot] : count_algo();
     const int parts = plan ? plan->parts[slot] : 0;
     if (algo == KC_ALGO_PIVOT) return sct_launch_slot(slot, Wh, c, pv, col, heavy, heavy_words, s);
@@ -511,6 +523,9 @@ Ctx base_ctx(const CountArgs& a)
     c.adjp = nullptr;
     c.queue = nullptr;
     c.perm = nullptr;
+    c.core = nullptr;
+    c.core_lo = INT32_MAX;
+    c.core_tw = 0;
     c.q0 = c.q1 = 0;
     c.nitems = 0;
     c.qoff = 0;
@@ -614,10 +629,7 @@ kc_status count_launch(const kc_graph* g, const CountArgs& a, unsigned long long
                        uint32_t* heavy_scratch, int64_t heavy_words, cudaStream_t s)
 {
     Ctx base = base_ctx(a);
-    base.offp = g->offp;
-    base.adjp = g->adjp;
-    base.queue = g->queue;
-    base.perm = g->perm;
+    cc::set_graph(base, g);
     const kc_graph::Parts* parts = nullptr;
     if (a.nparts > 1) KC_TRY(graph_parts(g, a.nparts, s, &parts));
     const bool col = a.colours >= 2 || a.pair;  // one colour keeps every pair
@@ -867,13 +879,10 @@ kc_status tune(const kc_graph* const* gs, int ng, int k, bool pv, cudaStream_t s
     cc::GraphDesc* dd = nullptr;
     const int64_t per = 2LL * ng + 1;
     if (ng == 1) {
-        base.offp = gs[0]->offp;
-        base.adjp = gs[0]->adjp;
-        base.queue = gs[0]->queue;
-        base.perm = gs[0]->perm;
+        cc::set_graph(base, gs[0]);
     } else {
         std::vector<cc::GraphDesc> hd((size_t)ng);
-        for (int i = 0; i < ng; ++i) hd[(size_t)i] = {gs[i]->offp, gs[i]->adjp, gs[i]->queue, gs[i]->perm};
+        for (int i = 0; i < ng; ++i) hd[(size_t)i] = cc::desc_of(gs[i]);
         host_tables.assign((size_t)(per * kOwnerSlots), 0);
         for (int slot = 0; slot < kOwnerSlots; ++slot) {
             int64_t* hq0 = host_tables.data() + slot * per;

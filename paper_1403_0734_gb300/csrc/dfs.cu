@@ -656,95 +656,48 @@ __device__ unsigned long long compact_count(uint32_t C, int n, int need, const u
     return tot;
 }
 
-// Owners with 33..64 elements (two-word rows), one warp each, without shared
-// memory: lane j holds x_j and x_{j+32} and, as 64-bit words, their rows of
-// G+(u) -- built like the one-word class (each 32-entry chunk of Gamma+(x_i)
-// searched for both elements of every lane by shuffle binary search, four
-// rows' first chunks loaded together) -- then the compact search (cdfs)
-// counts the (k-1)-cliques on those registers.  No block barrier, no
-// per-owner set-up beyond the loads: these owners are too many and too small
-// for a CTA each.  NEED = 4 (k = 6): the candidate sets of the first level are
-// closed instead (close.cuh); Chung-Lu n = 1e6: 12.1 -> 2.8 ms, of which 2.0 ms
-// build the rows.
+// Owners with 33..64 elements (two-word rows), one warp each: lane j holds x_j
+// and x_{j+32} and, as 64-bit words, their rows of G+(u) (build_rows_small);
+// the compact search (cdfs) counts the (k-1)-cliques on those registers.  No
+// block barrier, no per-owner set-up beyond the loads: these owners are too
+// many and too small for a CTA each.  NEED = 4 (k = 6): the candidate sets of
+// the first level are closed instead (close.cuh); Chung-Lu n = 1e6: search 10
+// -> 0.7 ms.
+constexpr int kW2Take = 4;  // owners a warp takes per cursor step at most
+
 template <bool PV, bool COL, int NEED>
-__global__ void __launch_bounds__(256) k_count_w2(Ctx cb)
+__global__ void __launch_bounds__(256, 4) k_count_w2(Ctx cb, int take)
 {
     constexpr cl::TeamLayout tl = cl::team_layout(2, 2, 1);
     constexpr int kRS = 4;  // row stride of the copy in shared memory
     __shared__ __align__(16) char s_team[NEED ? 8 : 1][NEED ? tl.total : 16];
     __shared__ __align__(16) uint32_t s_rows[NEED ? 8 : 1][NEED ? 64 * kRS : 4];
     __shared__ unsigned long long s_pv[NEED && PV ? 8 : 1][64];
+    __shared__ cc::SmallBuf<2> s_buf[NEED ? 1 : 8];
+    static_assert(tl.total >= (int)sizeof(cc::SmallBuf<2>), "the rows are built in the team's place");
     const int lane = threadIdx.x & 31;
+    cc::SmallBuf<2>& sb = NEED ? *(cc::SmallBuf<2>*)s_team[threadIdx.x >> 5] : s_buf[threadIdx.x >> 5];
     const int need = cb.k - 1;  // vertices to choose inside G+(u)
-    for (;;) {
-        unsigned long long pos = 0;
-        if (lane == 0) pos = atomicAdd(cb.cursor, 1ull);
-        pos = __shfl_sync(kFull, pos, 0);
+    cc::TotalSum total(cb.total);
+    cc::Owners own(take);
+    while (own.next(cb, lane)) {
         Ctx c;
         int32_t r;
-        if (!cc::resolve(cb, (int64_t)pos, c, r)) break;
-        const int64_t b = c.offp[r];
-        const int d = (int)(c.offp[r + 1] - b);  // 33..64
-        const int32_t xa = lane < d ? c.adjp[b + lane] : INT_MAX;
-        const int32_t xb = lane + 32 < d ? c.adjp[b + 32 + lane] : INT_MAX;
+        int64_t b;
+        int d;  // 33..64
+        own.take(cb, lane, c, r, b, d);
+        const int32_t xs[2] = {lane < d ? c.adjp[b + lane] : INT_MAX, lane + 32 < d ? c.adjp[b + 32 + lane] : INT_MAX};
+        const int32_t xa = xs[0], xb = xs[1];
         const int32_t ur = COL ? c.perm[r] : 0;
-        uint32_t cola = 0, colb = 0;
+        uint32_t cols[2] = {0u, 0u};
         if (COL) {
-            if (lane < d) cola = cc::sample_label(c, ur, c.perm[xa]);
-            if (lane + 32 < d) colb = cc::sample_label(c, ur, c.perm[xb]);
+            if (lane < d) cols[0] = cc::sample_label(c, ur, c.perm[xa]);
+            if (lane + 32 < d) cols[1] = cc::sample_label(c, ur, c.perm[xb]);
         }
-        const int32_t maxL = __shfl_sync(kFull, xb, (d - 33) & 31);
-        const bool ha = lane < d - 1, hb = lane + 32 < d - 1;
-        const int64_t la0 = ha ? c.offp[xa] : 0, la1 = ha ? c.offp[xa + 1] : 0;
-        const int64_t lb0 = hb ? c.offp[xb] : 0, lb1 = hb ? c.offp[xb + 1] : 0;
-        unsigned long long u0 = 0, u1 = 0;  // upper rows of elements lane, lane + 32
-        for (int i0 = 0; i0 < d - 1; i0 += 4) {
-            int32_t y[4];
-            int64_t s0[4], s1[4];
-#pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                const int i = i0 + t;
-                const int64_t a0 = __shfl_sync(kFull, la0, i & 31), a1 = __shfl_sync(kFull, la1, i & 31);
-                const int64_t b0 = __shfl_sync(kFull, lb0, i & 31), b1 = __shfl_sync(kFull, lb1, i & 31);
-                s0[t] = i < 32 ? a0 : b0;
-                s1[t] = i < 32 ? a1 : b1;
-                if (i >= d - 1) s1[t] = s0[t];
-                const int64_t p = s0[t] + lane;
-                y[t] = p < s1[t] ? c.adjp[p] : INT_MAX;
-            }
-#pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                const int i = i0 + t;
-                if (i >= d - 1) break;
-                unsigned long long row = 0;
-                for (int64_t p0 = s0[t];;) {
-                    int la = 0, lb = 0;
-#pragma unroll
-                    for (int step = 16; step > 0; step >>= 1) {
-                        const int32_t ya = __shfl_sync(kFull, y[t], la + step - 1);
-                        if (ya < xa) la += step;
-                        const int32_t yb = __shfl_sync(kFull, y[t], lb + step - 1);
-                        if (yb < xb) lb += step;
-                    }
-                    const bool hit_a = __shfl_sync(kFull, y[t], la) == xa && lane > i && lane < d;
-                    const bool hit_b = __shfl_sync(kFull, y[t], lb) == xb && lane + 32 > i && lane + 32 < d;
-                    row |= (unsigned long long)__ballot_sync(kFull, hit_a) |
-                           ((unsigned long long)__ballot_sync(kFull, hit_b) << 32);
-                    p0 += 32;
-                    if (p0 >= s1[t] || __shfl_sync(kFull, y[t], 31) >= maxL) break;
-                    const int64_t p = p0 + lane;
-                    y[t] = p < s1[t] ? c.adjp[p] : INT_MAX;
-                }
-                if (COL) {
-                    const uint32_t ci = i < 32 ? __shfl_sync(kFull, cola, i & 31) : __shfl_sync(kFull, colb, i & 31);
-                    row &= (unsigned long long)__ballot_sync(kFull, cc::sample_keep(c, ur, ci, cola)) |
-                           ((unsigned long long)__ballot_sync(kFull, cc::sample_keep(c, ur, ci, colb)) << 32);
-                }
-                if (lane == (i & 31)) {
-                    if (i < 32) u0 = row; else u1 = row;
-                }
-            }
-        }
+        uint32_t rows[2][2];
+        cc::build_rows_small<2, COL>(c, xs, d, cols, ur, sb, lane, rows);
+        const unsigned long long u0 = ((unsigned long long)rows[0][1] << 32) | rows[0][0];  // upper rows of
+        const unsigned long long u1 = ((unsigned long long)rows[1][1] << 32) | rows[1][0];  // lane, lane + 32
         unsigned long long f0 = u0, f1 = u1;  // full rows (memberships, closing): add the transpose
         if (PV || NEED) {
             for (int j = 1; j < d; ++j) {
@@ -793,8 +746,8 @@ __global__ void __launch_bounds__(256) k_count_w2(Ctx cb)
             }
             __syncwarp();
         }
+        total.add(c.total, tot, lane);
         if (lane == 0) {
-            add_total(c.total, tot);
             if (c.po) c.po[r] = tot;
             if (PV && tot) atomicAdd(&c.pv[r], tot);
             if (c.work && wk) atomicAdd(c.work, wk);
@@ -804,6 +757,7 @@ __global__ void __launch_bounds__(256) k_count_w2(Ctx cb)
             if (a1 && lane + 32 < d) atomicAdd(&c.pv[xb], a1);
         }
     }
+    total.flush(lane);
 }
 
 // Chains below a first-level choice: level 0 holds C (elements above i1),
@@ -1200,9 +1154,9 @@ kc_status w2_launch(const cc::Ctx& c, bool pv, bool col, cudaStream_t s)
 {
     if (c.nitems <= 0) return KC_OK;
     auto go = [&](auto kern) -> kc_status {
-        const int grid =
-            (int)std::min<int64_t>((c.nitems + 7) / 8, (int64_t)num_sms() * cc::blocks_per_sm(kern, 256, 0));
-        kern<<<grid, 256, 0, s>>>(c);
+        const cc::OwnerSteps st =
+            cc::owner_steps(c.nitems, 8, (int64_t)num_sms() * cc::blocks_per_sm(kern, 256, 0), kW2Take);
+        kern<<<st.grid, 256, 0, s>>>(c, st.take);
         KC_LAUNCHED();
         return KC_OK;
     };

@@ -88,6 +88,12 @@ struct kc_graph {
     int64_t* offp = nullptr;   // [n+1] oriented CSR offsets, rank space
     int32_t* adjp = nullptr;   // [m]  oriented CSR columns (ranks), rows ascending
     int32_t* queue = nullptr;  // [n]  owners (ranks): bitmap class, then work estimate (see kc.h)
+    // Adjacency bitmap of the core, the last ranks of the order: bit y - core_lo
+    // of row x - core_lo set iff x and y (both >= core_lo) are adjacent; rows of
+    // core_tw words.  core_lo = INT32_MAX: none.
+    uint32_t* core = nullptr;
+    int32_t core_lo = INT32_MAX;
+    int32_t core_tw = 0;
     void* block = nullptr;     // one pool allocation holding the arrays above
     int64_t bytes = 0;
     // host statistics: valid once ready() has returned KC_OK

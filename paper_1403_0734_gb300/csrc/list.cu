@@ -385,10 +385,7 @@ kc_status list_run(const kc_graph* g, int k, unsigned flags, int32_t* buf, int64
                               s));
         KC_CK(cudaMemsetAsync(cursors, 0, kCursorWords * sizeof(unsigned long long), s));
         Ctx base;
-        base.offp = g->offp;
-        base.adjp = g->adjp;
-        base.queue = g->queue;
-        base.perm = g->perm;
+        cc::set_graph(base, g);
         base.qoff = 0;
         base.qstride = 1;
         base.gd = nullptr;

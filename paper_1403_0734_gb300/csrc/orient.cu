@@ -925,6 +925,37 @@ __global__ void k_validate(const int64_t* __restrict__ off, const int32_t* __res
     }
 }
 
+constexpr int kCoreMax = 16384;  // ranks in the core at most: a bitmap of 32 MiB, a quarter of the L2 cache
+
+// Ranks in the core of a graph of n vertices and m edges: no more than give a
+// bitmap of the size of the oriented lists (4 m bytes).  Chung-Lu n = 1e6, m =
+// 2e7: the top 16384 ranks hold 83 % of the list entries that a count reads
+// (95 % at 32768, but that bitmap is as large as the L2 cache).
+int64_t core_ranks(int32_t n, int64_t m)
+{
+    int64_t t = std::min<int64_t>(n, kCoreMax);
+    while (t > 128 && t * t > 32 * m) t -= std::max<int64_t>(1, t / 64);
+    return m > 0 ? std::min<int64_t>((t + 127) & ~(int64_t)127, kCoreMax) : 0;
+}
+
+// Both bits of every edge inside the core, a warp per row of the core.
+__global__ void __launch_bounds__(kThreads) k_core(const int64_t* __restrict__ offp, const int32_t* __restrict__ adjp,
+                                                   int32_t n, int64_t m, int32_t lo, int tw, uint32_t* __restrict__ core)
+{
+    const int lane = threadIdx.x & 31;
+    const int nw = (int)(gridDim.x * blockDim.x) >> 5;
+    for (int32_t r = lo + (int32_t)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); r < n; r += nw) {
+        const int64_t e = min(offp[r + 1], m);  // (a CSR that was not symmetric: rows may be missing)
+        const int x = r - lo;
+        for (int64_t p = offp[r] + lane; p < e; p += 32) {
+            const int y = adjp[p] - lo;
+            if (y <= x || y >= n - lo) continue;
+            atomicOr(&core[(int64_t)x * tw + (y >> 5)], 1u << (y & 31));
+            atomicOr(&core[(int64_t)y * tw + (x >> 5)], 1u << (x & 31));
+        }
+    }
+}
+
 __global__ void k_zero_offset(int64_t* offp) { offp[0] = 0; }
 
 int grid_for(int64_t work, int per_block, int max_blocks)
@@ -987,7 +1018,14 @@ kc_status orient(const int64_t* off_in, const int32_t* adj_in, int32_t n, int64_
 
     // resident arrays: one pool block
     {
-        const size_t bytes = 5 * carve_bytes<int32_t>(nn) + carve_bytes<int64_t>(n1) + carve_bytes<int32_t>(m);
+        const int64_t ranks = core_ranks(n, m);
+        if (ranks > 0) {
+            g->core_lo = (int32_t)std::max<int64_t>(0, n - ranks);
+            g->core_tw = (int32_t)(ranks / 32);
+        }
+        const int64_t core_words = ranks > 0 ? (int64_t)(n - g->core_lo) * g->core_tw : 0;
+        const size_t bytes = 5 * carve_bytes<int32_t>(nn) + carve_bytes<int64_t>(n1) + carve_bytes<int32_t>(m) +
+                             (ranks > 0 ? carve_bytes<uint32_t>(core_words) : 0);
         KC_TRY(pool_alloc(&g->block, bytes, s));
         char* p = (char*)g->block;
         g->rank = carve<int32_t>(p, nn);
@@ -997,6 +1035,10 @@ kc_status orient(const int64_t* off_in, const int32_t* adj_in, int32_t n, int64_
         g->queue = carve<int32_t>(p, nn);
         g->offp = carve<int64_t>(p, n1);
         g->adjp = carve<int32_t>(p, m);
+        if (ranks > 0) {
+            g->core = carve<uint32_t>(p, core_words);
+            KC_CK(cudaMemsetAsync(g->core, 0, (size_t)core_words * sizeof(uint32_t), s));
+        }
         g->bytes = (int64_t)bytes;
     }
     g->hstats = stats_slot_get();
@@ -1116,6 +1158,13 @@ kc_status orient(const int64_t* off_in, const int32_t* adj_in, int32_t n, int64_
         k_rows_long<<<sms * 2, kThreads, 0, s>>>(off, g->perm, g->dplus, g->offp, tmp, m, g->adjp, kA, sort_rows,
                                                  rows_cap, ctl);
         KC_LAUNCHED();
+
+        // adjacency bitmap of the last ranks, for the builds of G+(u)
+        if (g->core) {
+            k_core<<<grid_for((int64_t)(n - g->core_lo) * 32, kThreads, sms * 8), kThreads, 0, s>>>(
+                g->offp, g->adjp, n, m, g->core_lo, g->core_tw, g->core);
+            KC_LAUNCHED();
+        }
 
         // a5: owner queue (one pass on the 8-bit key; stable, so ties by rank)
         {

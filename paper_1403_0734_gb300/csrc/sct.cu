@@ -60,6 +60,7 @@ __device__ __forceinline__ unsigned long long binom(int n, int r, bool* ovf)
 template <bool PV, bool COL>
 __global__ void __launch_bounds__(256) k_sct_w1(Ctx cb)
 {
+    __shared__ cc::SmallBuf<1> s_buf[8];
     const int lane = threadIdx.x & 31;
     const int need = cb.k - 1;  // clique vertices inside G+(u)
     for (;;) {
@@ -76,7 +77,11 @@ __global__ void __launch_bounds__(256) k_sct_w1(Ctx cb)
         const int32_t ur = COL ? c.perm[r] : 0;
         if (COL && lane < d) col = cc::sample_label(c, ur, c.perm[x]);
         if (COL) col = cc::class_flag_w1(c, col, d, c.k - 1, lane);
-        const uint32_t up = cc::build_rows_w1<COL>(c, x, d, col, ur, lane);
+        const int32_t xs[1] = {x};
+        const uint32_t cols[1] = {col};
+        uint32_t rows[1][1];
+        cc::build_rows_small<1, COL>(c, xs, d, cols, ur, s_buf[threadIdx.x >> 5], lane, rows);
+        const uint32_t up = rows[0][0];
         const uint32_t A = up | cc::lower_rows_w1(up, d, lane);  // N(lane) inside G+(u)
 
         const bool cw = c.work != nullptr;

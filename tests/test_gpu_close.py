@@ -72,3 +72,12 @@ def test_close_closed_forms(kc, parts, k):
     t, pv, _ = counts(kc, G, k)
     q = elementary(parts, k)
     assert t == q and np.all(pv == q * k // sum(parts))
+
+
+@pytest.mark.parametrize("k", [4, 5, 6])
+def test_batch_of_wide_graphs(kc, k):
+    # owners of every class in several graphs of one launch sequence
+    graphs = [kcgen.random_small(n, p, 31 * n) for n, p in ((300, 0.5), (40, 0.9), (520, 0.35), (200, 0.6), (90, 0.8))]
+    Gs = [kc.orient(g.off, g.adj) for g in graphs]
+    assert kc.count_batch(Gs, k) == [kc.count(G, k)[0] for G in Gs]
+    assert kc.count(Gs[4], k)[0] == oracle.count(graphs[4], k)[0]
