@@ -92,6 +92,33 @@ __device__ __forceinline__ unsigned long long leaf2_w1(uint32_t C, uint32_t up, 
     return (unsigned long long)__reduce_add_sync(kFull, e);
 }
 
+// Triangles inside C, the last two levels at once: lane v walks the members a
+// of C adjacent to it and counts popc(C & N(v) & N(a)).  Without memberships N
+// is the upper row (each triangle at its lowest vertex); with them the whole
+// row, which gives twice the triangles through v, its increment.  A row of
+// G+(u) has few elements in such sets, so this takes a handful of steps where
+// a step per element of C took all of them (one-word class, 8192 power-law
+// graphs, k = 4: see build_rows_small for the whole).
+template <bool PV>
+__device__ __forceinline__ unsigned long long leaf3_w1(uint32_t C, uint32_t up, uint32_t A, int lane,
+                                                       unsigned long long& pvl, unsigned long long* wk)
+{
+    const uint32_t row = PV ? A : up;
+    const uint32_t mine = ((C >> lane) & 1u) ? C & row : 0u;
+    uint32_t left = __popc(mine) >= 2 ? mine : 0u, cnt = 0;
+    for (;;) {
+        const uint32_t act = __ballot_sync(kFull, left != 0u);
+        if (act == 0u) break;
+        const uint32_t ra = __shfl_sync(kFull, row, (__ffs(left) - 1) & 31);
+        if (left) cnt += (uint32_t)__popc(mine & ra);
+        left &= left - 1u;
+        if (wk) *wk += (unsigned long long)__popc(act);
+    }
+    if (PV) pvl += cnt >> 1;
+    const uint32_t sum = __reduce_add_sync(kFull, cnt);
+    return PV ? sum / 6u : sum;
+}
+
 constexpr int kW1Take = 8;  // owners a warp takes per cursor step at most
 
 template <bool PV, bool COL>
@@ -104,80 +131,86 @@ __global__ void __launch_bounds__(256) k_count_w1(Ctx cb, int take)
     cc::TotalSum total(cb.total);
     cc::Owners own(take);
     while (own.next(cb, lane)) {
-        Ctx c;
+        cc::Gr g;
         int32_t r;
         int64_t b;
         int d;
-        own.take(cb, lane, c, r, b, d);
-        int32_t xs[1] = {lane < d ? c.adjp[b + lane] : INT_MAX};
+        own.take(cb, g, r, b, d);
+        int32_t xs[1] = {lane < d ? g.adjp[b + lane] : INT_MAX};
         const int32_t x = xs[0];
         uint32_t cols[1] = {0u};
-        const int32_t ur = COL ? c.perm[r] : 0;
-        if (COL && lane < d) cols[0] = cc::sample_label(c, ur, c.perm[x]);
-        if (COL) cols[0] = cc::class_flag_w1(c, cols[0], d, r0, lane);
+        const int32_t ur = COL ? cb.perm[r] : 0;
+        if (COL && lane < d) cols[0] = cc::sample_label(cb, ur, cb.perm[x]);
+        if (COL) cols[0] = cc::class_flag_w1(cb, cols[0], d, r0, lane);
 
         // (b) rows
         uint32_t rows[1][1];
-        cc::build_rows_small<1, COL>(c, xs, d, cols, ur, sb, lane, rows);
+        cc::build_rows_small<1, COL>(cb, g, xs, d, cols, ur, sb, lane, rows);
         const uint32_t up = rows[0][0];
         const uint32_t A = PV ? (up | cc::lower_rows_w1(up, d, lane)) : up;
 
-        // (c) depth-first search; level t's state of the chain is kept in lane t
+        // (c) depth-first search down to three missing vertices; level t's state
+        // of the chain is kept in lane t.  Of a candidate set C only the
+        // elements with enough higher neighbours in C are visited.
         unsigned long long tot = 0, pvl = 0, wk = 0;
-        const bool cw = c.work != nullptr;
+        unsigned long long* wkp = cb.work ? &wk : nullptr;
         const uint32_t C1 = d >= 32 ? kFull : ((1u << d) - 1u);
         if (r0 == 2) {
             tot = leaf2_w1<PV>(C1, up, A, lane, pvl);
-            if (cw) wk += (unsigned long long)__popc(C1) * (PV ? 2 : 1);
+            if (wkp) wk += (unsigned long long)__popc(C1) * (PV ? 2 : 1);
+        } else if (r0 == 3) {
+            tot = leaf3_w1<PV>(C1, up, A, lane, pvl, wkp);
         } else {
-            uint32_t st_rem = 0;
+            uint32_t st_C = 0, st_it = 0;
             int st_e = 0;
             unsigned long long st_sub = 0;
             int t = 0;
-            uint32_t cur = C1;
+            uint32_t C = C1;
+            uint32_t it = __ballot_sync(kFull, ((C >> lane) & 1u) && __popc(C & up) >= r0 - 1);
             unsigned long long cur_sub = 0;
             for (;;) {
-                if (cur == 0) {
+                if (it == 0) {
                     if (t == 0) break;
                     const unsigned long long sdone = cur_sub;
                     --t;
-                    cur = __shfl_sync(kFull, st_rem, t);
+                    C = __shfl_sync(kFull, st_C, t);
+                    it = __shfl_sync(kFull, st_it, t);
                     const int pe = __shfl_sync(kFull, st_e, t);
                     cur_sub = __shfl_sync(kFull, st_sub, t) + sdone;
                     if (PV && lane == pe) pvl += sdone;
                     continue;
                 }
-                const int e = __ffs(cur) - 1;
-                cur &= cur - 1u;
-                const uint32_t Cn = cur & __shfl_sync(kFull, up, e);
-                const int need = r0 - t - 1;
-                if (cw) wk += 1;
-                if (__popc(Cn) < need) continue;
-                if (need == 2) {
-                    if (cw) wk += (unsigned long long)__popc(Cn) * (PV ? 2 : 1);
-                    const unsigned long long E = leaf2_w1<PV>(Cn, up, A, lane, pvl);
+                const int e = __ffs(it) - 1;
+                it &= it - 1u;
+                const uint32_t Cn = C & __shfl_sync(kFull, up, e);
+                const int need = r0 - t - 1;  // vertices to choose in Cn
+                if (wkp) wk += 1;
+                if (need == 3) {
+                    const unsigned long long E = leaf3_w1<PV>(Cn, up, A, lane, pvl, wkp);
                     tot += E;
                     cur_sub += E;
                     if (PV && lane == e) pvl += E;
                 } else {
                     if (lane == t) {
-                        st_rem = cur;
+                        st_C = C;
+                        st_it = it;
                         st_e = e;
                         st_sub = cur_sub;
                     }
                     ++t;
-                    cur = Cn;
+                    C = Cn;
+                    it = __ballot_sync(kFull, ((C >> lane) & 1u) && __popc(C & up) >= need - 1);
                     cur_sub = 0;
                 }
             }
         }
-        total.add(c.total, tot, lane);
+        total.add(g.total, tot, lane);
         if (lane == 0) {
-            if (c.po) c.po[r] = tot;
-            if (PV && tot) atomicAdd(&c.pv[r], tot);
-            if (cw && wk) atomicAdd(c.work, wk);
+            if (cb.po) cb.po[r] = tot;
+            if (PV && tot) atomicAdd(&cb.pv[r], tot);
+            if (wk) atomicAdd(cb.work, wk);
         }
-        if (PV && lane < d && pvl) atomicAdd(&c.pv[x], pvl);
+        if (PV && lane < d && pvl) atomicAdd(&cb.pv[x], pvl);
     }
     total.flush(lane);
 }

@@ -220,38 +220,69 @@ struct TotalSum {
     }
 };
 
+// One owner's graph, for the one-warp kernels (sampling labels need the
+// caller's ids, Ctx::perm: single graphs only).
+struct Gr {
+    const int64_t* offp;
+    const int32_t* adjp;
+    const uint32_t* core;
+    int32_t core_lo, core_tw;
+    unsigned long long* total;
+};
+
 // Owners for one-warp kernels, `take` (at most 32) per cursor step: their
-// offsets and sizes are fetched together, a lane each.
+// graphs, ranks, offsets and sizes are fetched together, a lane each.
 struct Owners {
     int take_n;
     __device__ __forceinline__ explicit Owners(int n) : take_n(n) {}
-    unsigned long long pos = 0;
     int have = 0, at = 0;
+    int32_t rank = 0;
+    int graph = 0, deg = 0;
     int64_t off = 0;
-    int deg = 0;
     // Whether there is another owner; the same in every lane.
     __device__ __forceinline__ bool next(const Ctx& cb, int lane)
     {
         if (at < have) return true;
+        unsigned long long pos = 0;
         if (lane == 0) pos = atomicAdd(cb.cursor, (unsigned long long)take_n);
         pos = __shfl_sync(kFull, pos, 0);
         if ((int64_t)pos >= cb.nitems) return false;
         at = 0;
         have = (int)min((int64_t)take_n, cb.nitems - (int64_t)pos);
         if (lane < have) {
-            Ctx c;
-            int32_t rank;
-            resolve(cb, (int64_t)pos + lane, c, rank);
-            off = c.offp[rank];
-            deg = (int)(c.offp[rank + 1] - off);
+            const int64_t item = (int64_t)pos + lane;
+            const int64_t* offp;
+            if (cb.ng == 0) {
+                rank = cb.queue[cb.q0 + cb.qoff + item * cb.qstride];
+                offp = cb.offp;
+            } else {
+                int lo = 0, hi = cb.ng;  // largest g with gpre[g] <= item
+                while (hi - lo > 1) {
+                    const int mid = (lo + hi) >> 1;
+                    if (cb.gpre[mid] <= item) lo = mid; else hi = mid;
+                }
+                graph = lo;
+                rank = cb.gd[lo].queue[cb.gq0[lo] + (item - cb.gpre[lo])];
+                offp = cb.gd[lo].offp;
+            }
+            off = offp[rank];
+            deg = (int)(offp[rank + 1] - off);
         }
         return true;
     }
-    __device__ __forceinline__ void take(const Ctx& cb, int lane, Ctx& c, int32_t& r, int64_t& b, int& d)
+    __device__ __forceinline__ void take(const Ctx& cb, Gr& g, int32_t& r, int64_t& b, int& d)
     {
-        resolve(cb, (int64_t)pos + at, c, r);  // (c: its graph's pointers; always an item)
+        r = __shfl_sync(kFull, rank, at);
         b = __shfl_sync(kFull, off, at);
         d = __shfl_sync(kFull, deg, at);
+        const int gi = __shfl_sync(kFull, graph, at);
+        const GraphDesc* p = cb.gd + gi;
+        g.offp = cb.ng ? p->offp : cb.offp;
+        g.adjp = cb.ng ? p->adjp : cb.adjp;
+        g.core = cb.ng ? p->core : cb.core;
+        g.core_lo = cb.ng ? p->core_lo : cb.core_lo;
+        g.core_tw = cb.ng ? p->core_tw : cb.core_tw;
+        g.total = cb.total + 2 * gi;
         ++at;
     }
 };
@@ -289,7 +320,7 @@ struct SmallBuf {
 constexpr int kHashTries = 8;
 
 template <int W, bool COL>
-__device__ __forceinline__ void build_rows_small(const Ctx& c, const int32_t (&x)[W], int d, const uint32_t (&col)[W],
+__device__ __forceinline__ void build_rows_small(const Ctx& c, const Gr& g, const int32_t (&x)[W], int d, const uint32_t (&col)[W],
                                                  int32_t ur, SmallBuf<W>& sb, int lane, uint32_t (&up)[W][W])
 {
     constexpr int kShift = W == 1 ? 22 : 21;
@@ -301,10 +332,10 @@ __device__ __forceinline__ void build_rows_small(const Ctx& c, const int32_t (&x
     for (int h = 0; h < W; ++h) {
         const int j = lane + 32 * h;
         sb.x[j] = x[h];
-        inside[h] = __ballot_sync(kFull, j < d && x[h] >= c.core_lo);
-        const bool need = j < d - 1 && x[h] < c.core_lo && !(COL && class_filter_on(c) && (col[h] & kSkipLabel));  // (small colour class)
-        s0[h] = need ? c.offp[x[h]] : 0;
-        len[h] = need ? (int)(c.offp[x[h] + 1] - s0[h]) : 0;
+        inside[h] = __ballot_sync(kFull, j < d && x[h] >= g.core_lo);
+        const bool need = j < d - 1 && x[h] < g.core_lo && !(COL && class_filter_on(c) && (col[h] & kSkipLabel));  // (small colour class)
+        s0[h] = need ? g.offp[x[h]] : 0;
+        len[h] = need ? (int)(g.offp[x[h] + 1] - s0[h]) : 0;
         if (d > 32 * h) maxL = __shfl_sync(kFull, x[h], (d - 1 - 32 * h) & 31);
 #pragma unroll
         for (int w = 0; w < W; ++w) up[h][w] = 0u;
@@ -344,7 +375,7 @@ __device__ __forceinline__ void build_rows_small(const Ctx& c, const int32_t (&x
 #pragma unroll
         for (int w = 0; w < W; ++w) m[w] = 0u;
         // rel: this lane's first entry of the step, relative to the list's start
-        const int32_t* list = c.adjp + b;
+        const int32_t* list = g.adjp + b;
         for (int rel = 4 * sub - (int)(b & 3); rel < n; rel += 16) {
             const int4 y = *(const int4*)(list + rel);
             const int32_t ys[4] = {y.x, y.y, y.z, y.w};
@@ -382,9 +413,9 @@ __device__ __forceinline__ void build_rows_small(const Ctx& c, const int32_t (&x
             int lo = 0, hi = len[h];
             while (lo < hi) {
                 const int mid = (lo + hi) >> 1;
-                if (c.adjp[s0[h] + mid] < xe) lo = mid + 1; else hi = mid;
+                if (g.adjp[s0[h] + mid] < xe) lo = mid + 1; else hi = mid;
             }
-            if (lo < len[h] && c.adjp[s0[h] + lo] == xe) {
+            if (lo < len[h] && g.adjp[s0[h] + lo] == xe) {
                 if (W == 1 || e < 32) up[h][0] |= 1u << (e & 31);
                 else up[h][W - 1] |= 1u << (e & 31);
             }
@@ -394,7 +425,7 @@ __device__ __forceinline__ void build_rows_small(const Ctx& c, const int32_t (&x
     if (nlist < d - 1) {
         int off[W];
 #pragma unroll
-        for (int h = 0; h < W; ++h) off[h] = ((inside[h] >> lane) & 1u) ? x[h] - c.core_lo : 0;
+        for (int h = 0; h < W; ++h) off[h] = ((inside[h] >> lane) & 1u) ? x[h] - g.core_lo : 0;
 #pragma unroll 1
         for (int i0 = nlist; i0 < d - 1; i0 += 4) {
             uint32_t v[4][W];
@@ -403,7 +434,7 @@ __device__ __forceinline__ void build_rows_small(const Ctx& c, const int32_t (&x
                 const int i = min(i0 + t, d - 1);
                 int xi = __shfl_sync(kFull, off[0], i & 31);
                 if (W == 2 && i >= 32) xi = __shfl_sync(kFull, off[W - 1], i & 31);
-                const uint32_t* row = c.core + (int64_t)xi * c.core_tw;
+                const uint32_t* row = g.core + (int64_t)xi * g.core_tw;
 #pragma unroll
                 for (int h = 0; h < W; ++h) {
                     const int j = lane + 32 * h;

@@ -547,8 +547,53 @@ __device__ __forceinline__ unsigned long long cleaf2(unsigned long long C, unsig
     return (unsigned long long)__reduce_add_sync(kFull, e);
 }
 
+// Triangles inside the compact set C, the last two levels at once (as
+// leaf3_w1 in count.cu: lanes walk their vertices' members of C).
+template <bool PV>
+__device__ __forceinline__ unsigned long long cleaf3(unsigned long long C, unsigned long long u0,
+                                                     unsigned long long u1, unsigned long long f0,
+                                                     unsigned long long f1, int lane, unsigned long long& a0,
+                                                     unsigned long long& a1, unsigned long long* wk)
+{
+    const unsigned long long r0 = PV ? f0 : u0, r1 = PV ? f1 : u1;
+    const unsigned long long m0 = ((C >> lane) & 1ull) ? C & r0 : 0ull, m1 = ((C >> (lane + 32)) & 1ull) ? C & r1 : 0ull;
+    unsigned long long l0 = __popcll(m0) >= 2 ? m0 : 0ull, l1 = __popcll(m1) >= 2 ? m1 : 0ull;
+    unsigned c0 = 0, c1 = 0;
+    for (;;) {
+        const uint32_t act0 = __ballot_sync(kFull, l0 != 0ull), act1 = __ballot_sync(kFull, l1 != 0ull);
+        if ((act0 | act1) == 0u) break;
+        if (act0) {
+            const unsigned long long ra = crow(r0, r1, (__ffsll((long long)l0) - 1) & 63);
+            if (l0) c0 += (unsigned)__popcll(m0 & ra);
+            l0 &= l0 - 1ull;
+        }
+        if (act1) {
+            const unsigned long long ra = crow(r0, r1, (__ffsll((long long)l1) - 1) & 63);
+            if (l1) c1 += (unsigned)__popcll(m1 & ra);
+            l1 &= l1 - 1ull;
+        }
+        if (wk) *wk += 2ull * (unsigned long long)(__popc(act0) + __popc(act1));
+    }
+    if (PV) {
+        a0 += c0 >> 1;
+        a1 += c1 >> 1;
+    }
+    const unsigned sum = __reduce_add_sync(kFull, c0 + c1);
+    return PV ? sum / 6u : sum;
+}
+
+// The elements of C with at least `nd` higher neighbours in C.
+__device__ __forceinline__ unsigned long long cvisit(unsigned long long C, unsigned long long u0,
+                                                     unsigned long long u1, int nd, int lane)
+{
+    const bool v0 = ((C >> lane) & 1ull) && __popcll(C & u0) >= nd;
+    const bool v1 = ((C >> (lane + 32)) & 1ull) && __popcll(C & u1) >= nd;
+    return (unsigned long long)__ballot_sync(kFull, v0) | ((unsigned long long)__ballot_sync(kFull, v1) << 32);
+}
+
 // Cliques of `need` (>= 2) vertices chosen from the n-vertex compact graph
 // (upper rows u, full rows f in per-vertex mode), with memberships in a0/a1.
+// Chains end with three vertices missing.
 template <bool PV>
 __device__ unsigned long long cdfs(unsigned long long u0, unsigned long long u1, unsigned long long f0,
                                    unsigned long long f1, int n, int need, int lane, unsigned long long& a0,
@@ -559,15 +604,17 @@ __device__ unsigned long long cdfs(unsigned long long u0, unsigned long long u1,
         if (wk) *wk += (unsigned long long)n * (PV ? 4 : 2);
         return cleaf2<PV>(all, u0, u1, f0, f1, lane, a0, a1);
     }
-    unsigned long long tot = 0, cur = all, cur_sub = 0;
-    unsigned long long st_rem = 0, st_sub = 0;
+    if (need == 3) return cleaf3<PV>(all, u0, u1, f0, f1, lane, a0, a1, wk);
+    unsigned long long tot = 0, C = all, it = cvisit(all, u0, u1, need - 1, lane), cur_sub = 0;
+    unsigned long long st_C = 0, st_it = 0, st_sub = 0;
     int st_e = 0, t = 0;
     for (;;) {
-        if (cur == 0ull) {
+        if (it == 0ull) {
             if (t == 0) break;
             const unsigned long long sdone = cur_sub;
             --t;
-            cur = __shfl_sync(kFull, st_rem, t);
+            C = __shfl_sync(kFull, st_C, t);
+            it = __shfl_sync(kFull, st_it, t);
             const int pe = __shfl_sync(kFull, st_e, t);
             cur_sub = __shfl_sync(kFull, st_sub, t) + sdone;
             if (PV && lane == (pe & 31)) {
@@ -575,15 +622,13 @@ __device__ unsigned long long cdfs(unsigned long long u0, unsigned long long u1,
             }
             continue;
         }
-        const int e = __ffsll((long long)cur) - 1;
-        cur &= cur - 1ull;
-        const unsigned long long Cn = cur & crow(u0, u1, e);
-        const int nd = need - t - 1;
+        const int e = __ffsll((long long)it) - 1;
+        it &= it - 1ull;
+        const unsigned long long Cn = C & crow(u0, u1, e);
+        const int nd = need - t - 1;  // vertices to choose in Cn
         if (wk) *wk += 2;
-        if (__popcll(Cn) < nd) continue;
-        if (nd == 2) {
-            if (wk) *wk += (unsigned long long)__popcll(Cn) * (PV ? 4 : 2);
-            const unsigned long long E = cleaf2<PV>(Cn, u0, u1, f0, f1, lane, a0, a1);
+        if (nd == 3) {
+            const unsigned long long E = cleaf3<PV>(Cn, u0, u1, f0, f1, lane, a0, a1, wk);
             tot += E;
             cur_sub += E;
             if (PV && lane == (e & 31)) {
@@ -591,12 +636,14 @@ __device__ unsigned long long cdfs(unsigned long long u0, unsigned long long u1,
             }
         } else {
             if (lane == t) {
-                st_rem = cur;
+                st_C = C;
+                st_it = it;
                 st_e = e;
                 st_sub = cur_sub;
             }
             ++t;
-            cur = Cn;
+            C = Cn;
+            it = cvisit(C, u0, u1, nd - 1, lane);
             cur_sub = 0;
         }
     }
@@ -681,21 +728,21 @@ __global__ void __launch_bounds__(256, 4) k_count_w2(Ctx cb, int take)
     cc::TotalSum total(cb.total);
     cc::Owners own(take);
     while (own.next(cb, lane)) {
-        Ctx c;
+        cc::Gr g;
         int32_t r;
         int64_t b;
         int d;  // 33..64
-        own.take(cb, lane, c, r, b, d);
-        const int32_t xs[2] = {lane < d ? c.adjp[b + lane] : INT_MAX, lane + 32 < d ? c.adjp[b + 32 + lane] : INT_MAX};
+        own.take(cb, g, r, b, d);
+        const int32_t xs[2] = {lane < d ? g.adjp[b + lane] : INT_MAX, lane + 32 < d ? g.adjp[b + 32 + lane] : INT_MAX};
         const int32_t xa = xs[0], xb = xs[1];
-        const int32_t ur = COL ? c.perm[r] : 0;
+        const int32_t ur = COL ? cb.perm[r] : 0;
         uint32_t cols[2] = {0u, 0u};
         if (COL) {
-            if (lane < d) cols[0] = cc::sample_label(c, ur, c.perm[xa]);
-            if (lane + 32 < d) cols[1] = cc::sample_label(c, ur, c.perm[xb]);
+            if (lane < d) cols[0] = cc::sample_label(cb, ur, cb.perm[xa]);
+            if (lane + 32 < d) cols[1] = cc::sample_label(cb, ur, cb.perm[xb]);
         }
         uint32_t rows[2][2];
-        cc::build_rows_small<2, COL>(c, xs, d, cols, ur, sb, lane, rows);
+        cc::build_rows_small<2, COL>(cb, g, xs, d, cols, ur, sb, lane, rows);
         const unsigned long long u0 = ((unsigned long long)rows[0][1] << 32) | rows[0][0];  // upper rows of
         const unsigned long long u1 = ((unsigned long long)rows[1][1] << 32) | rows[1][0];  // lane, lane + 32
         unsigned long long f0 = u0, f1 = u1;  // full rows (memberships, closing): add the transpose
@@ -711,7 +758,7 @@ __global__ void __launch_bounds__(256, 4) k_count_w2(Ctx cb, int take)
         unsigned long long a0 = 0, a1 = 0, wk = 0;
         unsigned long long tot = 0;
         if constexpr (NEED == 0) {
-            tot = cdfs<PV>(u0, u1, f0, f1, d, need, lane, a0, a1, c.work ? &wk : nullptr);
+            tot = cdfs<PV>(u0, u1, f0, f1, d, need, lane, a0, a1, cb.work ? &wk : nullptr);
         } else {
             // the candidate set of every first-level vertex closed on a compact
             // copy, out of the rows in shared memory
@@ -733,28 +780,28 @@ __global__ void __launch_bounds__(256, 4) k_count_w2(Ctx cb, int take)
                     if (PV) mine[t.pos[j]] += K;
                 };
                 const unsigned long long sub =
-                    n <= 32 ? cl::close_set<1, (NEED ? NEED : 4), 32>(t, n, A, kRS, 2, lane, 0, c.work ? &wk : nullptr, credit)
-                            : cl::close_set<2, (NEED ? NEED : 4), 32>(t, n, A, kRS, 2, lane, 0, c.work ? &wk : nullptr, credit);
+                    n <= 32 ? cl::close_set<1, (NEED ? NEED : 4), 32>(t, n, A, kRS, 2, lane, 0, cb.work ? &wk : nullptr, credit)
+                            : cl::close_set<2, (NEED ? NEED : 4), 32>(t, n, A, kRS, 2, lane, 0, cb.work ? &wk : nullptr, credit);
                 tot += sub;
                 if (PV && sub && lane == 0) mine[e1] += sub;
                 __syncwarp();
             }
-            if (c.work) wk = warp_sum64(wk);
+            if (cb.work) wk = warp_sum64(wk);
             if (PV) {
                 a0 = mine[lane];
                 a1 = mine[lane + 32];
             }
             __syncwarp();
         }
-        total.add(c.total, tot, lane);
+        total.add(g.total, tot, lane);
         if (lane == 0) {
-            if (c.po) c.po[r] = tot;
-            if (PV && tot) atomicAdd(&c.pv[r], tot);
-            if (c.work && wk) atomicAdd(c.work, wk);
+            if (cb.po) cb.po[r] = tot;
+            if (PV && tot) atomicAdd(&cb.pv[r], tot);
+            if (cb.work && wk) atomicAdd(cb.work, wk);
         }
         if (PV) {
-            if (a0 && lane < d) atomicAdd(&c.pv[xa], a0);
-            if (a1 && lane + 32 < d) atomicAdd(&c.pv[xb], a1);
+            if (a0 && lane < d) atomicAdd(&cb.pv[xa], a0);
+            if (a1 && lane + 32 < d) atomicAdd(&cb.pv[xb], a1);
         }
     }
     total.flush(lane);

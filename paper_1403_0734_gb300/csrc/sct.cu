@@ -80,7 +80,8 @@ __global__ void __launch_bounds__(256) k_sct_w1(Ctx cb)
         const int32_t xs[1] = {x};
         const uint32_t cols[1] = {col};
         uint32_t rows[1][1];
-        cc::build_rows_small<1, COL>(c, xs, d, cols, ur, s_buf[threadIdx.x >> 5], lane, rows);
+        const cc::Gr g{c.offp, c.adjp, c.core, c.core_lo, c.core_tw, c.total};
+        cc::build_rows_small<1, COL>(c, g, xs, d, cols, ur, s_buf[threadIdx.x >> 5], lane, rows);
         const uint32_t up = rows[0][0];
         const uint32_t A = up | cc::lower_rows_w1(up, d, lane);  // N(lane) inside G+(u)
 
