@@ -421,38 +421,51 @@ __device__ __forceinline__ void build_rows_small(const Ctx& c, const Gr& g, cons
             }
         }
     }
-    // rows of the core's elements, four gathers in flight
+    // rows of the core's elements, four at a time: every lane reads its own
+    // elements' words of the row (lanes without one read word 0 and mask it), and
+    // four lanes keep the ballots; what does not belong to an upper row of the
+    // core is masked once at the end
     if (nlist < d - 1) {
+        uint32_t word[W], bit[W], val[W][W];
         int off[W];
 #pragma unroll
-        for (int h = 0; h < W; ++h) off[h] = ((inside[h] >> lane) & 1u) ? x[h] - g.core_lo : 0;
+        for (int h = 0; h < W; ++h) {
+            const bool in = (inside[h] >> lane) & 1u;
+            off[h] = in ? x[h] - g.core_lo : 0;
+            word[h] = (uint32_t)off[h] >> 5;
+            bit[h] = in ? 1u << (off[h] & 31) : 0u;
+#pragma unroll
+            for (int w = 0; w < W; ++w) val[h][w] = 0u;
+        }
 #pragma unroll 1
-        for (int i0 = nlist; i0 < d - 1; i0 += 4) {
+        for (int i0 = nlist & ~3; i0 < d - 1; i0 += 4) {
             uint32_t v[4][W];
 #pragma unroll
             for (int t = 0; t < 4; ++t) {
-                const int i = min(i0 + t, d - 1);
-                int xi = __shfl_sync(kFull, off[0], i & 31);
-                if (W == 2 && i >= 32) xi = __shfl_sync(kFull, off[W - 1], i & 31);
+                int xi = __shfl_sync(kFull, off[0], (i0 + t) & 31);
+                if (W == 2 && i0 >= 32) xi = __shfl_sync(kFull, off[W - 1], (i0 + t) & 31);
                 const uint32_t* row = g.core + (int64_t)xi * g.core_tw;
 #pragma unroll
-                for (int h = 0; h < W; ++h) {
-                    const int j = lane + 32 * h;
-                    v[t][h] = j > i && j < d ? row[off[h] >> 5] : 0u;
+                for (int h = 0; h < W; ++h) v[t][h] = row[word[h]];
+            }
+            const bool mine = (unsigned)(lane ^ (i0 & 31)) < 4u;
+#pragma unroll
+            for (int h = 0; h < W; ++h) {
+                const uint32_t b0 = __ballot_sync(kFull, v[0][h] & bit[h]), b1 = __ballot_sync(kFull, v[1][h] & bit[h]);
+                const uint32_t b2 = __ballot_sync(kFull, v[2][h] & bit[h]), b3 = __ballot_sync(kFull, v[3][h] & bit[h]);
+                const uint32_t w = lane & 2 ? (lane & 1 ? b3 : b2) : (lane & 1 ? b1 : b0);
+                if (mine) {
+                    if (W == 1 || i0 < 32) val[0][h] = w;
+                    else val[W - 1][h] = w;
                 }
             }
+        }
 #pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                const int i = i0 + t;
+        for (int h = 0; h < W; ++h) {
+            const int j = lane + 32 * h;
+            if (j < nlist || j >= d) continue;
 #pragma unroll
-                for (int h = 0; h < W; ++h) {
-                    const uint32_t w = __ballot_sync(kFull, (v[t][h] >> (off[h] & 31)) & 1u);
-                    if (i < d - 1 && lane == (i & 31)) {
-                        if (W == 1 || i < 32) up[0][h] = w;
-                        else up[W - 1][h] = w;
-                    }
-                }
-            }
+            for (int w = h; w < W; ++w) up[h][w] = w == h ? val[h][w] & mask_above(lane) : val[h][w];
         }
     }
     if (COL) {

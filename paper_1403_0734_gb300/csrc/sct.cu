@@ -39,11 +39,28 @@ namespace {
 using cc::add_total;
 using cc::Ctx;
 
+// C(n, r) for n <= 64, 0 <= r <= n / 2: all below 2^64 (C(64,32) < 2^61).
+struct Pascal {
+    unsigned long long c[65][33];
+    constexpr Pascal() : c{}
+    {
+        for (int n = 0; n <= 64; ++n) {
+            c[n][0] = 1;
+            for (int r = 1; r <= 32 && r <= n; ++r)
+                c[n][r] = c[n - 1][r - 1] + (r <= n - 1 && r <= 32 ? c[n - 1][r] : 0);
+        }
+    }
+};
+__device__ const Pascal g_pascal = Pascal();
+
 // C(n, r) for 0 <= r, exact; sets *ovf when the value does not fit 64 bits.
+// Up to n = 64 (every node of the one- and two-word classes) from the table:
+// the 128-bit divisions cost more than the rest of such an owner's tree.
 __device__ __forceinline__ unsigned long long binom(int n, int r, bool* ovf)
 {
     if (r < 0 || n < 0 || r > n) return 0ull;
     if (r > n - r) r = n - r;
+    if (n <= 64) return g_pascal.c[n][r];
     unsigned __int128 c = 1;
     for (int i = 1; i <= r; ++i) {
         c = c * (unsigned __int128)(n - r + i) / (unsigned __int128)i;
@@ -63,6 +80,7 @@ __global__ void __launch_bounds__(256) k_sct_w1(Ctx cb)
     __shared__ cc::SmallBuf<1> s_buf[8];
     const int lane = threadIdx.x & 31;
     const int need = cb.k - 1;  // clique vertices inside G+(u)
+    cc::TotalSum total(cb.total);
     for (;;) {
         unsigned long long pos = 0;
         if (lane == 0) pos = atomicAdd(cb.cursor, 1ull);
@@ -189,8 +207,8 @@ __global__ void __launch_bounds__(256) k_sct_w1(Ctx cb)
                 Pm = fPm | (1u << fp);
             }
         }
+        total.add(c.total, tot, lane);
         if (lane == 0) {
-            add_total(c.total, tot);
             if (ovf) atomicAdd(&c.total[1], 1ull);
             if (c.po) c.po[r] = tot;
             if (PV && tot) atomicAdd(&c.pv[r], tot);
@@ -198,6 +216,7 @@ __global__ void __launch_bounds__(256) k_sct_w1(Ctx cb)
         }
         if (PV && lane < d && pvl) atomicAdd(&c.pv[x], pvl);
     }
+    total.flush(lane);
 }
 
 // ------------------------------------------------- wider owners (warp each)
@@ -225,7 +244,8 @@ __host__ __device__ inline WLayout make_wlayout(int W, int RS, int need, bool pv
     return l;
 }
 
-template <bool PV, bool COL, bool HEAVY>
+// TWO: the two-word class, rows built in registers (build_rows_small).
+template <bool PV, bool COL, bool HEAVY, bool TWO>
 __global__ void __launch_bounds__(256) k_sct_warp(Ctx cb, int W, uint32_t* gscratch, int64_t slot_words)
 {
     extern __shared__ __align__(16) uint32_t smem[];
@@ -244,6 +264,8 @@ __global__ void __launch_bounds__(256) k_sct_warp(Ctx cb, int W, uint32_t* gscra
     uint32_t* fr = base + lay.fr;
     uint32_t* cur = base + lay.cur;
     const uint32_t lt = (1u << lane) - 1u;
+    __shared__ cc::SmallBuf<2> s_buf[TWO ? 8 : 1];
+    cc::TotalSum total(cb.total);
 
     for (;;) {
         unsigned long long pos = 0;
@@ -262,11 +284,38 @@ __global__ void __launch_bounds__(256) k_sct_warp(Ctx cb, int W, uint32_t* gscra
             if (COL) sCol[j] = cc::sample_label(c, ur, c.perm[xj]);
             if (PV) sPV[j] = 0ull;
         }
-        for (int64_t j = lane; j < (int64_t)d * RS; j += 32) sA[j] = 0u;
+        if (!TWO)
+            for (int64_t j = lane; j < (int64_t)d * RS; j += 32) sA[j] = 0u;
         for (int w = lane; w < Wd; w += 32) cur[w] = w < (d >> 5) ? kFull : ((1u << (d & 31)) - 1u);
         __syncwarp();
         if (COL) cc::class_flags_smem<false>(c, sCol, d, c.k - 1, lane, 32);
-        cc::build_rows<true, COL>(c, sL, sCol, d, sA, RS, 0, 1, lane, ur);
+        if (TWO) {
+            const int32_t xs[2] = {lane < d ? sL[lane] : INT_MAX, lane + 32 < d ? sL[lane + 32] : INT_MAX};
+            const uint32_t cols[2] = {COL && lane < d ? sCol[lane] : 0u, COL && lane + 32 < d ? sCol[lane + 32] : 0u};
+            const cc::Gr g{c.offp, c.adjp, c.core, c.core_lo, c.core_tw, c.total};
+            uint32_t up[2][2];
+            cc::build_rows_small<2, COL>(c, g, xs, d, cols, ur, s_buf[wid], lane, up);
+            const unsigned long long u0 = ((unsigned long long)up[0][1] << 32) | up[0][0];
+            const unsigned long long u1 = ((unsigned long long)up[1][1] << 32) | up[1][0];
+            unsigned long long f0 = u0, f1 = u1;  // add the transpose
+            for (int j = 1; j < d; ++j) {
+                const unsigned long long colj = (unsigned long long)__ballot_sync(kFull, (u0 >> j) & 1ull) |
+                                                ((unsigned long long)__ballot_sync(kFull, (u1 >> j) & 1ull) << 32);
+                if (lane == (j & 31)) {
+                    if (j < 32) f0 |= colj; else f1 |= colj;
+                }
+            }
+            if (lane < d) {
+                sA[lane * RS] = (uint32_t)f0;
+                sA[lane * RS + 1] = (uint32_t)(f0 >> 32);
+            }
+            if (lane + 32 < d) {
+                sA[(lane + 32) * RS] = (uint32_t)f1;
+                sA[(lane + 32) * RS + 1] = (uint32_t)(f1 >> 32);
+            }
+        } else {
+            cc::build_rows<true, COL>(c, sL, sCol, d, sA, RS, 0, 1, lane, ur);
+        }
         __syncwarp();
 
         const bool cw = c.work != nullptr;
@@ -460,8 +509,8 @@ __global__ void __launch_bounds__(256) k_sct_warp(Ctx cb, int W, uint32_t* gscra
             }
             __syncwarp();
         }
+        total.add(c.total, tot, lane);
         if (lane == 0) {
-            add_total(c.total, tot);
             if (ovf) atomicAdd(&c.total[1], 1ull);
             if (c.po) c.po[r] = tot;
             if (PV && tot) atomicAdd(&c.pv[r], tot);
@@ -474,6 +523,7 @@ __global__ void __launch_bounds__(256) k_sct_warp(Ctx cb, int W, uint32_t* gscra
             }
         __syncwarp();
     }
+    total.flush(lane);
 }
 
 template <bool PV, bool COL>
@@ -489,7 +539,7 @@ kc_status launch_slot_sct(int slot, int Wh, const Ctx& c, uint32_t* heavy, int64
         const int NW = (int)std::min<int64_t>(4, slots);
         const int64_t warps = std::min<int64_t>(slots, c.nitems);
         const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(warps / NW, (int64_t)sms * 8));
-        k_sct_warp<PV, COL, true><<<grid, NW * 32, 0, s>>>(c, Wh, heavy, lay.total);
+        k_sct_warp<PV, COL, true, false><<<grid, NW * 32, 0, s>>>(c, Wh, heavy, lay.total);
         KC_LAUNCHED();
         return KC_OK;
     }
@@ -505,7 +555,7 @@ kc_status launch_slot_sct(int slot, int Wh, const Ctx& c, uint32_t* heavy, int64
     const size_t per_warp = (size_t)lay.total * 4;
     const int NW = (int)std::max<size_t>(1, std::min<size_t>(8, (size_t)(100 * 1024) / per_warp));
     const size_t smem = per_warp * NW;
-    auto kern = k_sct_warp<PV, COL, false>;
+    auto kern = W == 2 ? k_sct_warp<PV, COL, false, true> : k_sct_warp<PV, COL, false, false>;
     KC_CK(cc::allow_smem(kern, smem));
     const int64_t ctas = (c.nitems + NW - 1) / NW;
     const int grid = (int)std::min<int64_t>(ctas, (int64_t)sms * cc::blocks_per_sm(kern, NW * 32, smem));
