@@ -518,7 +518,8 @@ kc_status launch_slot_dfs(int slot, int Wh, const Ctx& c, uint32_t* heavy, int64
     const int W = slot_words(slot);
     if (W == 2 && parts <= 1 && !(PV && COL) && dfs_reg_supported(k))
         return w2_launch(c, PV, COL, s);  // a warp per owner, rows in registers
-    if (k == 4 && W >= 4) return quad_launch(c, W, 32 * Wh, PV, COL, s);  // triangles of G+(u), edge by edge
+    if ((k == 4 && W >= 4) || (k == 5 && W == 4))
+        return quad_launch(c, W, 32 * Wh, PV, COL, s);  // triangles or 4-cliques of G+(u), edge by edge
     if (dfs_reg_supported(k)) return dfs_reg_launch(c, W, 32 * Wh, PV, COL, sc, parts, s);  // register-resident search
     const int NW = warps_for_width(W);
     const Layout lay = make_layout(W, W + 1, NW, levels, PV, COL);

@@ -709,7 +709,8 @@ __device__ unsigned long long compact_count(uint32_t C, int n, int need, const u
 // block barrier, no per-owner set-up beyond the loads: these owners are too
 // many and too small for a CTA each.  NEED = 4 (k = 6): the candidate sets of
 // the first level are closed instead (close.cuh); Chung-Lu n = 1e6: search 10
-// -> 0.7 ms.
+// -> 0.7 ms.  NEED = 3 (k = 5): the 4-cliques of G+(u) edge by edge as in quad.cu,
+// four lanes to a row, rows in shared memory; 1.63 -> 0.64 ms, builds included.
 constexpr int kW2Take = 4;  // owners a warp takes per cursor step at most
 
 template <bool PV, bool COL, int NEED>
@@ -717,13 +718,13 @@ __global__ void __launch_bounds__(256, 4) k_count_w2(Ctx cb, int take)
 {
     constexpr cl::TeamLayout tl = cl::team_layout(2, 2, 1);
     constexpr int kRS = 4;  // row stride of the copy in shared memory
-    __shared__ __align__(16) char s_team[NEED ? 8 : 1][NEED ? tl.total : 16];
+    __shared__ __align__(16) char s_team[NEED == 4 ? 8 : 1][NEED == 4 ? tl.total : 16];
     __shared__ __align__(16) uint32_t s_rows[NEED ? 8 : 1][NEED ? 64 * kRS : 4];
     __shared__ unsigned long long s_pv[NEED && PV ? 8 : 1][64];
-    __shared__ cc::SmallBuf<2> s_buf[NEED ? 1 : 8];
+    __shared__ cc::SmallBuf<2> s_buf[NEED == 4 ? 1 : 8];
     static_assert(tl.total >= (int)sizeof(cc::SmallBuf<2>), "the rows are built in the team's place");
     const int lane = threadIdx.x & 31;
-    cc::SmallBuf<2>& sb = NEED ? *(cc::SmallBuf<2>*)s_team[threadIdx.x >> 5] : s_buf[threadIdx.x >> 5];
+    cc::SmallBuf<2>& sb = NEED == 4 ? *(cc::SmallBuf<2>*)s_team[threadIdx.x >> 5] : s_buf[threadIdx.x >> 5];
     const int need = cb.k - 1;  // vertices to choose inside G+(u)
     cc::TotalSum total(cb.total);
     cc::Owners own(take);
@@ -746,7 +747,7 @@ __global__ void __launch_bounds__(256, 4) k_count_w2(Ctx cb, int take)
         const unsigned long long u0 = ((unsigned long long)rows[0][1] << 32) | rows[0][0];  // upper rows of
         const unsigned long long u1 = ((unsigned long long)rows[1][1] << 32) | rows[1][0];  // lane, lane + 32
         unsigned long long f0 = u0, f1 = u1;  // full rows (memberships, closing): add the transpose
-        if (PV || NEED) {
+        if (PV || NEED == 4) {
             for (int j = 1; j < d; ++j) {
                 const unsigned long long colj = (unsigned long long)__ballot_sync(kFull, (u0 >> j) & 1ull) |
                                                 ((unsigned long long)__ballot_sync(kFull, (u1 >> j) & 1ull) << 32);
@@ -759,6 +760,70 @@ __global__ void __launch_bounds__(256, 4) k_count_w2(Ctx cb, int take)
         unsigned long long tot = 0;
         if constexpr (NEED == 0) {
             tot = cdfs<PV>(u0, u1, f0, f1, d, need, lane, a0, a1, cb.work ? &wk : nullptr);
+        } else if constexpr (NEED == 3) {
+            const int wid = threadIdx.x >> 5;
+            uint2* A = (uint2*)s_rows[wid];
+            unsigned long long* mine = s_pv[PV ? wid : 0];
+            const unsigned long long w0 = PV ? f0 : u0, w1 = PV ? f1 : u1;
+            A[lane] = make_uint2((uint32_t)w0, (uint32_t)(w0 >> 32));
+            A[lane + 32] = make_uint2((uint32_t)w1, (uint32_t)(w1 >> 32));
+            if (PV) mine[lane] = mine[lane + 32] = 0ull;
+            __syncwarp();
+            const uint32_t share = 0x11111111u << (lane & 3);
+            unsigned steps = 0;
+            // the lowest vertex of a 4-clique has three higher neighbours
+            const unsigned long long low = cvisit(~0ull, u0, u1, 3, lane);
+            for (int v0 = low ? 0 : d; v0 < d; v0 += 8) {
+                const int v = v0 + (lane >> 2);
+                const uint2 X = v < d ? A[v] : make_uint2(0u, 0u);
+                const uint32_t take = PV || ((low >> (v & 63)) & 1ull) ? share : 0u;
+                uint32_t b0 = X.x & take & (v < 32 ? mask_above(v) : 0u);
+                uint32_t b1 = X.y & take & (v < 32 ? kFull : mask_above(v - 32));
+                unsigned sum = 0;
+                while (b0 | b1) {
+                    int a;
+                    if (b0) {
+                        a = __ffs(b0) - 1;
+                        b0 &= b0 - 1u;
+                    } else {
+                        a = 31 + __ffs(b1);
+                        b1 &= b1 - 1u;
+                    }
+                    const uint2 Y = A[a];
+                    const uint32_t C0 = X.x & Y.x, C1 = X.y & Y.y;
+                    uint32_t l0 = C0, l1 = C1;
+                    unsigned co = 0;
+                    while (l0 | l1) {
+                        int e;
+                        if (l0) {
+                            e = __ffs(l0) - 1;
+                            l0 &= l0 - 1u;
+                        } else {
+                            e = 31 + __ffs(l1);
+                            l1 &= l1 - 1u;
+                        }
+                        const uint2 Z = A[e];
+                        co += (unsigned)(__popc(C0 & Z.x) + __popc(C1 & Z.y));
+                        ++steps;
+                    }
+                    if (PV && co) {
+                        co >>= 1;  // 4-cliques on the edge
+                        atomicAdd((uint32_t*)&mine[a], co);  // (at most 3 C(63,3): the low words do)
+                    }
+                    sum += co;
+                }
+                if (PV && sum) atomicAdd((uint32_t*)&mine[v], sum);
+                tot += sum;
+            }
+            tot = warp_sum64(tot);
+            if (PV) tot /= 6ull;
+            __syncwarp();
+            if (PV) {
+                a0 = mine[lane] / 3ull;
+                a1 = mine[lane + 32] / 3ull;
+            }
+            if (cb.work) wk = 2ull * __reduce_add_sync(kFull, steps);
+            __syncwarp();
         } else {
             // the candidate set of every first-level vertex closed on a compact
             // copy, out of the rows in shared memory
@@ -1210,6 +1275,10 @@ kc_status w2_launch(const cc::Ctx& c, bool pv, bool col, cudaStream_t s)
     if (c.k == 6 && g_complement) {
         if (pv) return col ? KC_ENOTSUP : go(k_count_w2<true, false, 4>);
         return col ? go(k_count_w2<false, true, 4>) : go(k_count_w2<false, false, 4>);
+    }
+    if (c.k == 5) {
+        if (pv) return col ? KC_ENOTSUP : go(k_count_w2<true, false, 3>);
+        return col ? go(k_count_w2<false, true, 3>) : go(k_count_w2<false, false, 3>);
     }
     if (pv) return col ? KC_ENOTSUP : go(k_count_w2<true, false, 0>);
     return col ? go(k_count_w2<false, true, 0>) : go(k_count_w2<false, false, 0>);

@@ -1,5 +1,14 @@
-// quad.cu -- k = 4 for owners of more than 64 elements (rows of 4..32 words).
+// quad.cu -- k = 4 for owners of more than 64 elements (rows of 4..32 words),
+// and k = 5 in the 4-word class.
 //
+// k = 5: q_{u,4} is the number of 4-cliques of G+(u); each edge v < a counts the
+// edges inside C = row v & row a, one row load for each b of C -- with whole
+// rows twice the 4-cliques on the edge, of which a vertex has three edges.
+// (Lists of the search's few elements per set cost more than these loops while
+// rows are 128 bits; from 8 words on sets are closed instead, close.cu.)
+// Chung-Lu n = 1e6, total: 1.43 -> 1.30 ms.
+//
+// k = 4:
 // q_{u,3} is the number of triangles of G+(u).  One CTA per owner builds the
 // bitmap rows in shared memory and walks the edges of G+(u), v < a, once: with
 // co = popc(row v & row a) over upper rows (no memberships) their sum is the
@@ -47,7 +56,7 @@ __host__ __device__ inline QLayout quad_layout(int D, int WM, bool pv, bool col)
     return l;
 }
 
-template <bool PV, bool COL, int WM>
+template <bool PV, bool COL, int WM, int K>
 __global__ void __launch_bounds__(WM <= 4 ? 128 : 256, WM <= 4 ? 8 : (WM <= 16 ? 4 : 1)) k_quad(Ctx cb, int D)
 {
     extern __shared__ __align__(16) uint32_t smem[];
@@ -84,7 +93,7 @@ __global__ void __launch_bounds__(WM <= 4 ? 128 : 256, WM <= 4 ? 8 : (WM <= 16 ?
             s_wk = 0ull;
         }
         __syncthreads();
-        if (COL) cc::class_flags_smem<true>(c, sCol, d, 3, threadIdx.x, blockDim.x);
+        if (COL) cc::class_flags_smem<true>(c, sCol, d, K - 1, threadIdx.x, blockDim.x);
         cc::SpanTable T{smem + lay.bits, (uint16_t*)(smem + lay.pre), 0, 0};
         if (sL[0] < c.core_lo) cc::span_table_build(T, sL, d, kSpanWords);  // (lists are read)
         cc::build_rows<PV, COL>(c, sL, sCol, d, sA, RS, wid, NW, lane, ur, &T);
@@ -116,13 +125,32 @@ __global__ void __launch_bounds__(WM <= 4 ? 128 : 256, WM <= 4 ? 8 : (WM <= 16 ?
                         bits &= bits - 1u;
                         const uint4* Ra = (const uint4*)(sA + a * RS);
                         uint32_t co = 0;
+                        if (K == 4) {
 #pragma unroll
-                        for (int q = 0; q < WM / 4; ++q) {
-                            if (q >= nq) continue;
-                            const uint4 x = Ra[q];
-                            const uint32_t z[4] = {X[4 * q] & x.x, X[4 * q + 1] & x.y, X[4 * q + 2] & x.z,
-                                                   X[4 * q + 3] & x.w};
-                            co += cl::popc_words<4>(z);
+                            for (int q = 0; q < WM / 4; ++q) {
+                                if (q >= nq) continue;
+                                const uint4 x = Ra[q];
+                                const uint32_t z[4] = {X[4 * q] & x.x, X[4 * q + 1] & x.y, X[4 * q + 2] & x.z,
+                                                       X[4 * q + 3] & x.w};
+                                co += cl::popc_words<4>(z);
+                            }
+                        } else {  // WM == 4
+                            const uint4 x = Ra[0];
+                            const uint32_t C[4] = {X[0] & x.x, X[1] & x.y, X[2] & x.z, X[3] & x.w};
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) {
+                                uint32_t left = C[q];
+#pragma unroll 1
+                                while (left) {
+                                    const int e = q * 32 + __ffs(left) - 1;
+                                    left &= left - 1u;
+                                    const uint4 y = *(const uint4*)(sA + e * RS);
+                                    const uint32_t z[4] = {C[0] & y.x, C[1] & y.y, C[2] & y.z, C[3] & y.w};
+                                    co += cl::popc_words<4>(z);
+                                    if (c.work) wk += 4u;
+                                }
+                            }
+                            if (PV) co >>= 1;  // 4-cliques on the edge
                         }
                         sum += co;
                         if (PV && co) atomicAdd(&acc[a], co);
@@ -140,8 +168,9 @@ __global__ void __launch_bounds__(WM <= 4 ? 128 : 256, WM <= 4 ? 8 : (WM <= 16 ?
             if (lane == 0 && wk) atomicAdd(&s_wk, wk);
         }
         __syncthreads();
-        // whole rows: every triangle was met on its three edges
-        const unsigned long long q = PV ? s_tot / 3ull : s_tot;
+        // whole rows: every triangle was met on its three edges, every 4-clique on
+        // its six; a vertex has two of the edges, or three
+        const unsigned long long q = PV ? s_tot / (K == 4 ? 3ull : 6ull) : s_tot;
         if (threadIdx.x == 0) {
             add_total(c.total, q);
             if (c.po) c.po[r] = q;
@@ -150,15 +179,15 @@ __global__ void __launch_bounds__(WM <= 4 ? 128 : 256, WM <= 4 ? 8 : (WM <= 16 ?
         }
         if (PV)
             for (int j = threadIdx.x; j < d; j += blockDim.x)
-                if (acc[j]) atomicAdd(&c.pv[sL[j]], (unsigned long long)(acc[j] >> 1));
+                if (acc[j]) atomicAdd(&c.pv[sL[j]], (unsigned long long)(acc[j] / (K == 4 ? 2u : 3u)));
         __syncthreads();
     }
 }
 
-template <bool PV, bool COL, int WM>
+template <bool PV, bool COL, int WM, int K>
 kc_status go(const Ctx& c, int D, cudaStream_t s)
 {
-    auto kern = k_quad<PV, COL, WM>;
+    auto kern = k_quad<PV, COL, WM, K>;
     const size_t smem = (size_t)quad_layout(D, WM, PV, COL).total * 4;
     const int threads = WM <= 4 ? 128 : 256;
     KC_CK(cc::allow_smem(kern, smem));
@@ -171,18 +200,20 @@ kc_status go(const Ctx& c, int D, cudaStream_t s)
 template <bool PV, bool COL>
 kc_status by_width(const Ctx& c, int W, int D, cudaStream_t s)
 {
+    if (c.k == 5) return W == 4 ? go<PV, COL, 4, 5>(c, D, s) : KC_ENOTSUP;
     switch (W) {
-    case 4: return go<PV, COL, 4>(c, D, s);
-    case 8: return go<PV, COL, 8>(c, D, s);
-    case 16: return go<PV, COL, 16>(c, D, s);
-    case 32: return go<PV, COL, 32>(c, D, s);
+    case 4: return go<PV, COL, 4, 4>(c, D, s);
+    case 8: return go<PV, COL, 8, 4>(c, D, s);
+    case 16: return go<PV, COL, 16, 4>(c, D, s);
+    case 32: return go<PV, COL, 32, 4>(c, D, s);
     }
     return KC_ENOTSUP;
 }
 
 }  // namespace
 
-// The class of W = 4, 8, 16 or 32 words at k = 4; dmax: no |Gamma+| is larger.
+// The class of W = 4, 8, 16 or 32 words at k = 4, of 4 words at k = 5; dmax: no
+// |Gamma+| is larger.
 kc_status quad_launch(const Ctx& c, int W, int dmax, bool pv, bool col, cudaStream_t s)
 {
     const int D = 32 * ((std::min(dmax, 32 * W) + 31) / 32);
