@@ -8,11 +8,14 @@
 // instructions more than for anything else), has shared memory for its own
 // sets only, and balances single sets instead of owners.
 // 4 words: an owner per CTA, rows in shared memory, a set per warp.
-// Chung-Lu n = 1e6, m = 2e7, against the pair search of dfs.cu: k = 6 with
-// memberships, 16-word class 325 -> 41 ms, 8-word 49 -> 8 ms, 4-word 17.4 -> 3.6
-// ms (issue slots 60-75 % busy); k = 5 total, 16-word class 11.1 -> 7.2 ms, 8
-// words 2.5 ms either way; colour estimate (c = 8, k = 6), 16-word class 8.1 ->
-// 1.5 ms.
+// Chung-Lu n = 1e6, m = 2e7, against the pair search of dfs.cu, tiles included:
+// k = 6 with memberships, 16-word class 325 -> 43 ms, 8-word 49 -> 6.7 ms,
+// 4-word 17.4 -> 2.5 ms (issue slots 60-75 % busy); k = 5 total, 16-word class
+// 11.9 -> 8.0 ms, 8-word 3.3 -> 3.1 ms; colour estimate (c = 8, k = 6), 16-word
+// class 9.0 -> 2.1 ms, 8-word 3.3 -> 1.4 ms.
+// Tried and not kept: the counts |X_v & X_a| over all a kept as binary digits
+// (bitwise row additions along X_v) instead of c intersections: widths 5, 6, 8
+// 3-9 % faster, widths 3 and 4 3-7 % slower, the whole k = 6 count 54.3 -> 52.8 ms.
 #include <algorithm>
 
 #include "close.cuh"
@@ -313,7 +316,9 @@ kc_status launch_bins(const Ctx& c, const Lists& L, int chunks, unsigned int* cu
 }  // namespace
 
 // Whether the closing kernels count k in the class of W words with `items`
-// owners (a list entry holds 22 bits of the owner's number).
+// owners (a list entry holds 22 bits of the owner's number).  k = 5 and 6: the
+// sets of the first level need three or four vertices there; both are faster
+// than the search (figures above), and k >= 7 would need five.
 bool close_supported(int W, int k, int64_t items) { return (W == 8 || W == 16) && (k == 5 || k == 6) && items < (1 << 22); }
 
 // Search pass of a split class over finished tiles (symmetric rows of RS = W

@@ -19,9 +19,10 @@
 //       lies in popc(C & row(e)) of them -- no per-clique work.
 //       Chain members and u are credited with the sub-tree totals.
 // Owners come from the queue (|Gamma+| descending) in classes by bitmap
-// width W = ceil(d/32): W = 1 runs one warp per owner with the rows in
-// registers; W in {2..32} one CTA per owner with the rows in shared memory;
-// wider owners use the same CTA code on a global-memory tile.
+// width W = ceil(d/32): W = 1 (here) and 2 (dfs.cu) run one warp per owner with
+// the rows in registers; W in {4..32} one CTA per owner with the rows in shared
+// memory (quad.cu, dfs.cu) or sets of many owners together (close.cu); wider
+// owners use this file's CTA code on a global-memory tile.
 #include <algorithm>
 #include <climits>
 #include <cstring>
@@ -121,6 +122,12 @@ __device__ __forceinline__ unsigned long long leaf3_w1(uint32_t C, uint32_t up, 
 }
 
 constexpr int kW1Take = 8;  // owners a warp takes per cursor step at most
+
+// Owners with at most 32 elements, one warp each.  Bound: the latency of their
+// short lists (a row is a list of a few dozen entries somewhere in the L2), so
+// rows are built eight lists at a time (build_rows_small), several owners come
+// from one cursor step, and one total leaves the warp at its end.  Chung-Lu n =
+// 1e6, k = 4 with memberships 2.76 -> 0.96 ms; SBM n = 2e6, k = 5 2.2 -> 0.91 ms.
 
 template <bool PV, bool COL>
 __global__ void __launch_bounds__(256) k_count_w1(Ctx cb, int take)
@@ -516,10 +523,15 @@ kc_status launch_slot_dfs(int slot, int Wh, const Ctx& c, uint32_t* heavy, int64
         return KC_OK;
     }
     const int W = slot_words(slot);
+    // A warp per owner, rows in registers, unless a plan splits owners (Chung-Lu
+    // n = 1e6, this class: k = 4 2.05 -> 0.45 ms, k = 6 12.1 -> 1.8 ms).
     if (W == 2 && parts <= 1 && !(PV && COL) && dfs_reg_supported(k))
-        return w2_launch(c, PV, COL, s);  // a warp per owner, rows in registers
+        return w2_launch(c, PV, COL, s);
+    // Triangles or 4-cliques of G+(u) edge by edge, at every width for k = 4 and
+    // at 4 words for k = 5 (both sides in quad.cu); k = 5 on wider rows closes
+    // sets instead: an edge's common neighbours are too many there to read each.
     if ((k == 4 && W >= 4) || (k == 5 && W == 4))
-        return quad_launch(c, W, 32 * Wh, PV, COL, s);  // triangles or 4-cliques of G+(u), edge by edge
+        return quad_launch(c, W, 32 * Wh, PV, COL, s);
     if (dfs_reg_supported(k)) return dfs_reg_launch(c, W, 32 * Wh, PV, COL, sc, parts, s);  // register-resident search
     const int NW = warps_for_width(W);
     const Layout lay = make_layout(W, W + 1, NW, levels, PV, COL);
@@ -535,7 +547,9 @@ kc_status launch_slot_dfs(int slot, int Wh, const Ctx& c, uint32_t* heavy, int64
 kc_status launch_slot(int slot, int Wh, const Ctx& c, bool pv, bool col, uint32_t* heavy, int64_t heavy_words,
                       Scratch* sc, const Plan* plan, cudaStream_t s)
 {
-    if (c.k == 3 && !col && tri_enabled()) {  // no bitmaps for k = 3 but in registers
+    // No bitmaps for k = 3 but in registers: up to 64 elements the rows built
+    // there beat the list search (Chung-Lu n = 1e6: 2.56 ms -> 0.33 + 0.92 ms).
+    if (c.k == 3 && !col && tri_enabled()) {
         if (slot_words(slot) == 1 || slot_words(slot) == 2)
             return pv ? launch_slot_dfs<true, false>(slot, Wh, c, heavy, heavy_words, sc, 1, s)
                       : launch_slot_dfs<false, false>(slot, Wh, c, heavy, heavy_words, sc, 1, s);

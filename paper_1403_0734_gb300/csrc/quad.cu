@@ -20,7 +20,8 @@
 // issue and shared-memory loads, about 40 instructions for 32 edges of a 16-word
 // row.  The general search (dfs.cu) spent 130 there: it listed each candidate
 // set's elements by rank before it read their rows.  Chung-Lu n = 1e6, m = 2e7,
-// with memberships, builds included: see quad_launch.
+// with memberships, builds included: 16 words 1.36 -> 0.94 ms, 8 words 1.15 ->
+// 0.63 ms, 4 words 1.14 -> 0.48 ms.
 #include <algorithm>
 
 #include "close.cuh"

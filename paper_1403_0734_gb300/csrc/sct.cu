@@ -55,7 +55,9 @@ __device__ const Pascal g_pascal = Pascal();
 
 // C(n, r) for 0 <= r, exact; sets *ovf when the value does not fit 64 bits.
 // Up to n = 64 (every node of the one- and two-word classes) from the table:
-// the 128-bit divisions cost more than the rest of such an owner's tree.
+// the 128-bit divisions cost more than the rest of such an owner's tree (SBM of
+// full blocks of 50, n = 2e6, k = 7 with memberships: 11.9 -> 4.55 ms with the
+// rows of the two-word class in registers).
 __device__ __forceinline__ unsigned long long binom(int n, int r, bool* ovf)
 {
     if (r < 0 || n < 0 || r > n) return 0ull;

@@ -2,7 +2,6 @@
 every row width of the copy (1..16 words), both sides of the flip to the
 complement, against the oracle where it can enumerate the cliques, against
 closed forms, and against the ordered search (KC_PARAM_COMPLEMENT = 0)."""
-import itertools
 from math import comb
 
 import numpy as np
@@ -81,3 +80,40 @@ def test_batch_of_wide_graphs(kc, k):
     Gs = [kc.orient(g.off, g.adj) for g in graphs]
     assert kc.count_batch(Gs, k) == [kc.count(G, k)[0] for G in Gs]
     assert kc.count(Gs[4], k)[0] == oracle.count(graphs[4], k)[0]
+
+
+@pytest.mark.parametrize("d", [31, 32, 33, 63, 64, 65, 127, 128, 129, 255, 256, 257, 511, 512, 513, 1000, 1024])
+@pytest.mark.parametrize("k", [3, 4, 5])
+def test_class_edges(kc, d, k):
+    # K_{d+1}: its first owner has d elements; then d elements of three colours and an apex
+    G = kc.orient(*_csr(kcgen.complete(d + 1)))
+    t, pv, _ = counts(kc, G, k)
+    assert t == comb(d + 1, k) and np.all(pv == comb(d, k - 1))
+    parts = (1,) + (d // 3, d // 3, d - 2 * (d // 3))
+    G = kc.orient(*_csr(kcgen.complete_multipartite(parts, shuffle_seed=d)))
+    assert counts(kc, G, k)[0] == elementary(parts, k)
+
+
+def _csr(g):
+    return g.off, g.adj
+
+
+@pytest.mark.parametrize("name", ["sbm", "chung_lu", "dense"])
+@pytest.mark.parametrize("k", [3, 4, 5, 6])
+def test_rows_from_lists_and_core(kc, name, k):
+    # rows read from sorted lists, from the bitmap of the last ranks, and from both within one owner
+    g = {"sbm": lambda: kcgen.sbm(2000, 50, 0.5, 50000, 4), "chung_lu": lambda: kcgen.chung_lu(3000, 40000, 2.1, 400.0, 5),
+         "dense": lambda: kcgen.random_small(120, 0.5, 6)}[name]()
+    G = kc.orient(*_csr(g))
+    t, pv, po = counts(kc, G, k)
+    ot, opo, opv = oracle.count(g, k, per_owner=True, per_vertex=True)
+    assert t == ot and np.array_equal(pv, opv) and np.array_equal(po, opo)
+    assert kc.count_batch([G, G], k) == [t, t]
+    for c in (1, 3):
+        s, _, spo = kc.estimate(G, k, c, 5, per_owner=True)
+        os_, _, ospo = oracle.estimate(g, k, c, 5, per_owner=True)
+        assert s == os_ and np.array_equal(spo, ospo)
+    if k <= 4:
+        rows = np.sort(kc.list_cliques(G, k), axis=1)
+        want = np.sort(oracle.list_cliques(g, k), axis=1)
+        assert np.array_equal(rows[np.lexsort(rows.T)], want[np.lexsort(want.T)])
