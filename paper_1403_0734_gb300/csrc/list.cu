@@ -192,6 +192,24 @@ __host__ __device__ inline LLayout make_llayout(int W, int RS, int NW, int level
     return l;
 }
 
+// Exclusive scan of cnt1[0..d), by one warp.
+__device__ void scan_counts(unsigned long long* cnt1, int d, int lane)
+{
+    unsigned long long carry = 0;
+    for (int b0 = 0; b0 < d; b0 += 32) {
+        const int j = b0 + lane;
+        const unsigned long long v = j < d ? cnt1[j] : 0ull;
+        unsigned long long incl = v;
+#pragma unroll
+        for (int s = 1; s < 32; s <<= 1) {
+            const unsigned long long x = __shfl_up_sync(kFull, incl, s);
+            if (lane >= s) incl += x;
+        }
+        if (j < d) cnt1[j] = carry + incl - v;
+        carry += __shfl_sync(kFull, incl, 31);
+    }
+}
+
 // One CTA per owner of the run: G+(u), per-x_i1 counts, their scan, writes.
 template <bool HEAVY>
 __global__ void __launch_bounds__(256) k_list(Ctx cb, int W, int levels, const unsigned long long* ooff,
@@ -247,21 +265,7 @@ __global__ void __launch_bounds__(256) k_list(Ctx cb, int W, int levels, const u
             if (lane == 0) cnt1[e1] = n1;
         }
         __syncthreads();
-        if (wid == 0) {  // exclusive scan of cnt1 by warp 0
-            unsigned long long carry = 0;
-            for (int b0 = 0; b0 < d; b0 += 32) {
-                const int j = b0 + lane;
-                const unsigned long long v = j < d ? cnt1[j] : 0ull;
-                unsigned long long incl = v;
-#pragma unroll
-                for (int s = 1; s < 32; s <<= 1) {
-                    const unsigned long long x = __shfl_up_sync(kFull, incl, s);
-                    if (lane >= s) incl += x;
-                }
-                if (j < d) cnt1[j] = carry + incl - v;
-                carry += __shfl_sync(kFull, incl, 31);
-            }
-        }
+        if (wid == 0) scan_counts(cnt1, d, lane);
         __syncthreads();
 
         // pass 2: write each sub-tree at its offset
@@ -283,17 +287,211 @@ __global__ void __launch_bounds__(256) k_list(Ctx cb, int W, int levels, const u
     }
 }
 
+template <int WM>
+__device__ __forceinline__ void load_row(const uint32_t* A, int e, uint32_t (&x)[WM])
+{
+    if (WM == 2) {
+        const uint2 v = ((const uint2*)A)[e];
+        x[0] = v.x;
+        x[1] = v.y;
+        return;
+    }
+#pragma unroll
+    for (int q = 0; q < WM / 4; ++q) {
+        const uint4 v = ((const uint4*)A)[e * (WM / 4) + q];
+        x[4 * q] = v.x;
+        x[4 * q + 1] = v.y;
+        x[4 * q + 2] = v.z;
+        x[4 * q + 3] = v.w;
+    }
+}
+
+// The cliques made of u, x_e1 and `need` vertices of row e1, in the order of
+// their chains: counted, or with WRITE stored from clique number pos on.  A
+// warp; every lane holds the whole candidate set, lane t the state of level t,
+// and lane j the caller's ids ids[q] of the elements 32 q + j.
+template <int WM, bool WRITE>
+__device__ unsigned long long walk(const uint32_t* A, const int32_t* sL, const int32_t (&ids)[WM], int e1, int need,
+                                   int32_t uid, int32_t* out, int kk, int64_t pos, int64_t lim, int lane)
+{
+    const bool quads = kk == 4 && ((uintptr_t)out & 15) == 0;  // a clique is one 128-bit store
+    const uint32_t lt = cc::mask_below(lane);
+    uint32_t C[WM], it[WM], st_C[WM], st_it[WM];
+    load_row<WM>(A, e1, C);
+    unsigned long long total = 0;
+    int32_t chid = sL[e1];  // lane t: id of the chain's t-th vertex
+    int t = 0;              // levels below x_e1
+#pragma unroll
+    for (int q = 0; q < WM; ++q) st_C[q] = st_it[q] = it[q] = 0u;
+
+    // elements of S as the last vertex
+    auto leaves = [&](const uint32_t (&S)[WM], int chain) {
+#pragma unroll
+        for (int q = 0; q < WM; ++q) {
+            if (S[q] == 0u) continue;
+            const int64_t row = pos + __popc(S[q] & lt);
+            const bool ok = ((S[q] >> lane) & 1u) && row < lim;  // rows past the run's buffer are never written
+            int32_t* o = out + row * kk;
+            if (quads) {
+                const int4 v = make_int4(uid, __shfl_sync(kFull, chid, 0), __shfl_sync(kFull, chid, 1), ids[q]);
+                if (ok) *(int4*)o = v;
+            } else {
+                for (int i = 0; i < chain; ++i) {
+                    const int32_t id = __shfl_sync(kFull, chid, i);
+                    if (ok) o[1 + i] = id;
+                }
+                if (ok) {
+                    o[0] = uid;
+                    o[kk - 1] = ids[q];
+                }
+            }
+            pos += __popc(S[q]);
+        }
+    };
+
+    if (need == 1) {
+        if (WRITE) {
+            leaves(C, 1);
+        } else {
+#pragma unroll
+            for (int q = 0; q < WM; ++q) total += (unsigned long long)__popc(C[q]);
+        }
+        return total;
+    }
+    bool enter = true;
+    for (;;) {
+        if (enter) {  // a new set: its elements that have enough neighbours above them in it
+            uint32_t sum = 0;
+#pragma unroll
+            for (int q = 0; q < WM; ++q) {
+                uint32_t n = 0;
+                if ((C[q] >> lane) & 1u) {
+                    uint32_t x[WM];
+                    load_row<WM>(A, q * 32 + lane, x);
+#pragma unroll
+                    for (int w = 0; w < WM; ++w) n += (uint32_t)__popc(C[w] & x[w]);
+                }
+                if (!WRITE) sum += n;
+                it[q] = __ballot_sync(kFull, n >= (uint32_t)(need - 1));
+            }
+            if (!WRITE && need == 2) {  // two vertices missing: the edges inside
+                total += (unsigned long long)__reduce_add_sync(kFull, sum);
+#pragma unroll
+                for (int q = 0; q < WM; ++q) it[q] = 0u;
+            }
+            enter = false;
+        }
+        int e = -1;
+#pragma unroll
+        for (int q = 0; q < WM; ++q)
+            if (e < 0 && it[q]) {
+                e = q * 32 + __ffs(it[q]) - 1;
+                it[q] &= it[q] - 1u;
+            }
+        if (e < 0) {
+            if (t == 0) break;
+            --t;
+            ++need;
+#pragma unroll
+            for (int q = 0; q < WM; ++q) {
+                C[q] = __shfl_sync(kFull, st_C[q], t);
+                it[q] = __shfl_sync(kFull, st_it[q], t);
+            }
+            continue;
+        }
+        uint32_t Cn[WM];
+        load_row<WM>(A, e, Cn);
+#pragma unroll
+        for (int q = 0; q < WM; ++q) Cn[q] &= C[q];
+        if (WRITE) {
+            const int32_t id = sL[e];
+            if (lane == t + 1) chid = id;
+            if (need == 2) {
+                leaves(Cn, t + 2);
+                continue;
+            }
+        }
+        if (lane == t) {
+#pragma unroll
+            for (int q = 0; q < WM; ++q) {
+                st_C[q] = C[q];
+                st_it[q] = it[q];
+            }
+        }
+        ++t;
+        --need;
+#pragma unroll
+        for (int q = 0; q < WM; ++q) C[q] = Cn[q];
+        enter = true;
+    }
+    return total;
+}
+
+// Owners of 33..32 WM elements, a CTA each: as k_list, with the sets and the
+// chain in registers (walk), the counts of pass 1 closed two levels early and a
+// clique of four ids stored at once.  Bound: the latency of an owner's chains,
+// a few hundred owners to a run.  k = 4, against k_list: a run of 325 owners of
+// two words 207 -> 59 us, of 3 owners of four words 263 -> 89 us; a listing of
+// 6.7e6 cliques with owners of eight words 1.49 -> 0.89 ms.  Wider owners stay
+// with k_list: sets in registers gained nothing there (0.357 against 0.362 ms
+// at k = 3, 16 words).
+template <int WM>
+__global__ void __launch_bounds__(256) k_list_reg(Ctx cb, const unsigned long long* ooff, int32_t* out, int64_t lim)
+{
+    constexpr int D = 32 * WM;
+    __shared__ __align__(16) uint32_t A[D * WM];
+    __shared__ int32_t sL[D];
+    __shared__ unsigned long long cnt1[D];
+    __shared__ long long s_item;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, NW = blockDim.x >> 5;
+    const int kk = cb.k, need = kk - 2;
+    for (;;) {
+        if (threadIdx.x == 0) s_item = (long long)atomicAdd(cb.cursor, 1ull);
+        __syncthreads();
+        const long long item = s_item;
+        Ctx c;
+        int32_t r;
+        if (!cc::resolve(cb, (int64_t)item, c, r)) break;
+        const int64_t b = c.offp[r];
+        const int d = (int)(c.offp[r + 1] - b);
+        const int32_t uid = c.perm[r];
+        const int64_t o = (int64_t)ooff[item];
+        for (int j = threadIdx.x; j < d; j += blockDim.x) sL[j] = c.adjp[b + j];
+        for (int j = threadIdx.x; j < d * WM; j += blockDim.x) A[j] = 0u;
+        __syncthreads();
+        cc::build_rows<false, false>(c, sL, nullptr, d, A, WM, wid, NW, lane);
+        __syncthreads();
+        for (int j = threadIdx.x; j < d; j += blockDim.x) sL[j] = c.perm[sL[j]];
+        __syncthreads();
+        int32_t ids[WM];
+#pragma unroll
+        for (int q = 0; q < WM; ++q) ids[q] = q * 32 + lane < d ? sL[q * 32 + lane] : 0;
+        for (int e1 = wid; e1 < d; e1 += NW) {
+            const unsigned long long n1 = walk<WM, false>(A, sL, ids, e1, need, uid, out, kk, 0, 0, lane);
+            if (lane == 0) cnt1[e1] = n1;
+        }
+        __syncthreads();
+        if (wid == 0) scan_counts(cnt1, d, lane);
+        __syncthreads();
+        for (int e1 = wid; e1 < d; e1 += NW)
+            walk<WM, true>(A, sL, ids, e1, need, uid, out, kk, o + (int64_t)cnt1[e1], lim, lane);
+        __syncthreads();
+    }
+}
+
 // Owners of at most 32 elements, a warp each, rows and chain in registers: the
 // cliques are met in the order the layout wants (x_i1, then the chains below it,
 // ascending), so one pass writes them from the owner's offset on.  k_list
 // counted every sub-tree first, with a CTA of one warp per owner: 754 us for
-// the 17,000 owners of a 20,000-vertex power-law graph at k = 4.
+// the 17,000 owners of a 20,000-vertex power-law graph at k = 4; here 108 us, 67
+// with a clique of four ids stored at once.
 __global__ void __launch_bounds__(256) k_list_w1(Ctx cb, const unsigned long long* ooff, int32_t* out, int64_t lim)
 {
     __shared__ cc::SmallBuf<1> s_buf[8];
     const int lane = threadIdx.x & 31;
     const uint32_t lt = cc::mask_below(lane);
     const int kk = cb.k, r0 = kk - 1;
+    const bool quads = kk == 4 && ((uintptr_t)out & 15) == 0;  // a clique is one 128-bit store
     for (;;) {
         unsigned long long item = 0;
         if (lane == 0) item = atomicAdd(cb.cursor, 1ull);
@@ -342,6 +540,14 @@ __global__ void __launch_bounds__(256) k_list_w1(Ctx cb, const unsigned long lon
             const int64_t row = pos + __popc(Cn & lt);
             const bool ok = ((Cn >> lane) & 1u) && row < lim;  // rows past the run's buffer are never written
             int32_t* o = out + row * kk;
+            if (quads) {
+                const int32_t i1 = __shfl_sync(kFull, id, __shfl_sync(kFull, st_e, 0));
+                const int32_t i2 = __shfl_sync(kFull, id, __shfl_sync(kFull, st_e, 1));
+                if (ok) *(int4*)o = make_int4(uid, i1, i2, id);
+                pos += __popc(Cn);
+                --t;
+                continue;
+            }
             for (int q = 0; q < t; ++q) {
                 const int32_t cid = __shfl_sync(kFull, id, __shfl_sync(kFull, st_e, q));
                 if (ok) o[1 + q] = cid;
@@ -531,6 +737,13 @@ kc_status list_run(const kc_graph* g, int k, unsigned flags, int32_t* buf, int64
                     const int grid = (int)std::min<int64_t>((c.nitems + 7) / 8,
                                                             (int64_t)sms * cc::blocks_per_sm(k_list_w1, 256, 0));
                     k_list_w1<<<grid, 256, 0, s>>>(c, off, dbuf, (int64_t)T);
+                    KC_LAUNCHED();
+                    continue;
+                }
+                if (W <= 8) {
+                    auto kern = W == 2 ? k_list_reg<2> : (W == 4 ? k_list_reg<4> : k_list_reg<8>);
+                    const int grid = (int)std::min<int64_t>(c.nitems, (int64_t)sms * cc::blocks_per_sm(kern, 256, 0));
+                    kern<<<grid, 256, 0, s>>>(c, off, dbuf, (int64_t)T);
                     KC_LAUNCHED();
                     continue;
                 }

@@ -117,3 +117,24 @@ def test_rows_from_lists_and_core(kc, name, k):
         rows = np.sort(kc.list_cliques(G, k), axis=1)
         want = np.sort(oracle.list_cliques(g, k), axis=1)
         assert np.array_equal(rows[np.lexsort(rows.T)], want[np.lexsort(want.T)])
+
+
+@pytest.mark.parametrize("k", [3, 4, 5])
+def test_listing_order_and_alignment(kc, k):
+    # owners of 1..8 words; the same rows in the same places of a buffer that starts off a 16-byte boundary
+    import torch
+    g = kcgen.random_small(300, 0.45, 8)
+    G = kc.orient(*_csr(g))
+    want = oracle.list_cliques(g, k)
+    buf = torch.empty((len(want) + 1) * k + 1, dtype=torch.int32, device="cuda")
+    got = []
+    for start in (0, 1):
+        buf.fill_(-1)
+        part = buf[start:]
+        assert kc.list_runs(G, k, lambda a: False, cap=len(want), device_buffer=part) == len(want)
+        rows = part[: len(want) * k].view(len(want), k).cpu().numpy()
+        assert int((part[len(want) * k :] == -1).all()) and (start == 0 or int(buf[0]) == -1)
+        got.append(rows.copy())
+    assert np.array_equal(got[0], got[1])
+    a, b = np.sort(got[0], axis=1), np.sort(want, axis=1)
+    assert np.array_equal(a[np.lexsort(a.T)], b[np.lexsort(b.T)])
