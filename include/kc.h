@@ -336,9 +336,9 @@ kc_status kc_count_batch(const kc_graph* const* gs, int ng, int k, unsigned flag
  *       follow from the degrees in G[C] and the rows of v's non-neighbours,
  *       so only the rows of non-neighbours are read.  It needs symmetric
  *       rows: per-vertex counts have them, and totals at k >= 6 in those
- *       classes take them for this (their memberships are dropped).  k = 5 and
- *       6 stop one level earlier where the rows are in split tiles (8 and 16
- *       words), and k = 6 in the 2- and 4-word classes too: a candidate set
+ *       classes take them for this (their memberships are dropped).  k = 6
+ *       stops one level earlier in the 2- to 16-word classes (8 and 16 words:
+ *       where the rows are in split tiles), k = 5 in the 16-word class: a candidate set
  *       that needs three or four vertices is closed on a compact copy of its
  *       subgraph, through the complement when that is the sparser side.  0:
  *       every such set is closed on its edges (one row read per neighbour) and

@@ -11,7 +11,7 @@
 // Chung-Lu n = 1e6, m = 2e7, against the pair search of dfs.cu, tiles included:
 // k = 6 with memberships, 16-word class 325 -> 43 ms, 8-word 49 -> 6.7 ms,
 // 4-word 17.4 -> 2.5 ms (issue slots 60-75 % busy); k = 5 total, 16-word class
-// 11.9 -> 8.0 ms, 8-word 3.3 -> 3.1 ms; colour estimate (c = 8, k = 6), 16-word
+// 11.9 -> 8.0 ms; colour estimate (c = 8, k = 6), 16-word
 // class 9.0 -> 2.1 ms, 8-word 3.3 -> 1.4 ms.
 // Tried and not kept: the counts |X_v & X_a| over all a kept as binary digits
 // (bitwise row additions along X_v) instead of c intersections: widths 5, 6, 8
@@ -317,9 +317,15 @@ kc_status launch_bins(const Ctx& c, const Lists& L, int chunks, unsigned int* cu
 
 // Whether the closing kernels count k in the class of W words with `items`
 // owners (a list entry holds 22 bits of the owner's number).  k = 5 and 6: the
-// sets of the first level need three or four vertices there; both are faster
-// than the search (figures above), and k >= 7 would need five.
-bool close_supported(int W, int k, int64_t items) { return (W == 8 || W == 16) && (k == 5 || k == 6) && items < (1 << 22); }
+// sets of the first level need three or four vertices there; k >= 7 would need
+// five.  k = 5 at 8 words stays with the search, whose sets are small there: whole
+// counts on Chung-Lu n = 1e6, search against closing, 13.6 / 13.9 ms and with
+// memberships 21.0 / 24.7; n = 3e5, 1.9 / 2.2 and 3.6 / 4.4 (R-MAT of scale 17: 2.8 /
+// 2.6 and 4.6 / 5.8).
+bool close_supported(int W, int k, int64_t items)
+{
+    return ((W == 16 && k == 5) || (W >= 8 && W <= 16 && k == 6)) && items < (1 << 22);
+}
 
 // Search pass of a split class over finished tiles (symmetric rows of RS = W
 // + 4 words, the candidate-set sizes in word W and their numbers by width in

@@ -529,9 +529,11 @@ kc_status launch_slot_dfs(int slot, int Wh, const Ctx& c, uint32_t* heavy, int64
     if (W == 2 && parts <= 1 && !(PV && COL) && dfs_reg_supported(k))
         return w2_launch(c, PV, COL, s);
     // Triangles or 4-cliques of G+(u) edge by edge, at every width for k = 4 and
-    // at 4 words for k = 5 (both sides in quad.cu); k = 5 on wider rows closes
-    // sets instead: an edge's common neighbours are too many there to read each.
-    if ((k == 4 && W >= 4) || (k == 5 && W == 4))
+    // at 4 words for k = 5 (both sides in quad.cu); on wider rows an edge's common
+    // neighbours are too many to read each (dfs.cu and close.cu).
+    // With memberships k = 5 reads whole rows, every 4-clique six times: the search
+    // is faster (Chung-Lu n = 1e6 21.0 -> 20.0 ms, R-MAT of scale 17 4.6 -> 3.2).
+    if ((k == 4 && W >= 4) || (k == 5 && W == 4 && !PV))
         return quad_launch(c, W, 32 * Wh, PV, COL, s);
     if (dfs_reg_supported(k)) return dfs_reg_launch(c, W, 32 * Wh, PV, COL, sc, parts, s);  // register-resident search
     const int NW = warps_for_width(W);

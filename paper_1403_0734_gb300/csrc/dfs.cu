@@ -1,5 +1,9 @@
 // dfs.cu -- ordered depth-first counter (Reduce 3, Alg. 1; Sec. 3) for owners
-// whose G+(u) bitmap fits in shared memory (|Gamma+(u)| <= 1024), k <= 8.
+// whose G+(u) bitmap fits in shared memory (|Gamma+(u)| <= 1024), k <= 8: every
+// class at k >= 7, the 32-word class at k = 5 and 6, and what other rules leave
+// (quad.cu: k = 4, and k = 5 totals at 4 words; close.cu: k = 5 at 16 words and
+// k = 6 at 8 and 16 words in split tiles, k = 6 at 4 words; k_count_w2 below: two
+// words).
 //
 // Same search as the generic kernel in count.cu -- chains x_i1 < x_i2 < ...
 // of G+(u) with candidate sets C_t = C_{t-1} & row(i_t), the last two levels

@@ -2,10 +2,9 @@
 // and k = 5 in the 4-word class.
 //
 // k = 5: q_{u,4} is the number of 4-cliques of G+(u); each edge v < a counts the
-// edges inside C = row v & row a, one row load for each b of C -- with whole
-// rows twice the 4-cliques on the edge, of which a vertex has three edges.
+// edges inside C = row v & row a, one row load for each b of C.  Totals only.
 // (Lists of the search's few elements per set cost more than these loops while
-// rows are 128 bits; from 8 words on sets are closed instead, close.cu.)
+// rows are 128 bits; 8 words stay with the search, 16 words close sets, close.cu.)
 // Chung-Lu n = 1e6, total: 1.43 -> 1.30 ms.
 //
 // k = 4:
@@ -57,7 +56,7 @@ __host__ __device__ inline QLayout quad_layout(int D, int WM, bool pv, bool col)
     return l;
 }
 
-template <bool PV, bool COL, int WM, int K>
+template <bool PV, bool COL, int WM, int K>  // K = 5: !PV, WM = 4
 __global__ void __launch_bounds__(WM <= 4 ? 128 : 256, WM <= 4 ? 8 : (WM <= 16 ? 4 : 1)) k_quad(Ctx cb, int D)
 {
     extern __shared__ __align__(16) uint32_t smem[];
@@ -151,7 +150,6 @@ __global__ void __launch_bounds__(WM <= 4 ? 128 : 256, WM <= 4 ? 8 : (WM <= 16 ?
                                     if (c.work) wk += 4u;
                                 }
                             }
-                            if (PV) co >>= 1;  // 4-cliques on the edge
                         }
                         sum += co;
                         if (PV && co) atomicAdd(&acc[a], co);
@@ -169,9 +167,8 @@ __global__ void __launch_bounds__(WM <= 4 ? 128 : 256, WM <= 4 ? 8 : (WM <= 16 ?
             if (lane == 0 && wk) atomicAdd(&s_wk, wk);
         }
         __syncthreads();
-        // whole rows: every triangle was met on its three edges, every 4-clique on
-        // its six; a vertex has two of the edges, or three
-        const unsigned long long q = PV ? s_tot / (K == 4 ? 3ull : 6ull) : s_tot;
+        // whole rows: every triangle was met on its three edges, a vertex has two of them
+        const unsigned long long q = PV ? s_tot / 3ull : s_tot;
         if (threadIdx.x == 0) {
             add_total(c.total, q);
             if (c.po) c.po[r] = q;
@@ -180,7 +177,7 @@ __global__ void __launch_bounds__(WM <= 4 ? 128 : 256, WM <= 4 ? 8 : (WM <= 16 ?
         }
         if (PV)
             for (int j = threadIdx.x; j < d; j += blockDim.x)
-                if (acc[j]) atomicAdd(&c.pv[sL[j]], (unsigned long long)(acc[j] / (K == 4 ? 2u : 3u)));
+                if (acc[j]) atomicAdd(&c.pv[sL[j]], (unsigned long long)(acc[j] / 2u));
         __syncthreads();
     }
 }
@@ -201,7 +198,10 @@ kc_status go(const Ctx& c, int D, cudaStream_t s)
 template <bool PV, bool COL>
 kc_status by_width(const Ctx& c, int W, int D, cudaStream_t s)
 {
-    if (c.k == 5) return W == 4 ? go<PV, COL, 4, 5>(c, D, s) : KC_ENOTSUP;
+    if (c.k == 5) {
+        if constexpr (PV) return KC_ENOTSUP;
+        else return W == 4 ? go<PV, COL, 4, 5>(c, D, s) : KC_ENOTSUP;
+    }
     switch (W) {
     case 4: return go<PV, COL, 4, 4>(c, D, s);
     case 8: return go<PV, COL, 8, 4>(c, D, s);
@@ -213,8 +213,8 @@ kc_status by_width(const Ctx& c, int W, int D, cudaStream_t s)
 
 }  // namespace
 
-// The class of W = 4, 8, 16 or 32 words at k = 4, of 4 words at k = 5; dmax: no
-// |Gamma+| is larger.
+// The class of W = 4, 8, 16 or 32 words at k = 4, of 4 words at k = 5 without
+// memberships; dmax: no |Gamma+| is larger.
 kc_status quad_launch(const Ctx& c, int W, int dmax, bool pv, bool col, cudaStream_t s)
 {
     const int D = 32 * ((std::min(dmax, 32 * W) + 31) / 32);
