@@ -16,8 +16,9 @@
 //       prefix of the queue for every k; inside the wider classes by the work
 //       estimate w(u) = sum over x in Gamma+(u) of |Gamma+(x)| (the Gamma+(x)
 //       entries Round 2 reads for u), descending; ties by rank.
-//   core: a symmetric bitmap of the edges among the last ranks (k_core), read
-//       by the counts instead of the lists of those vertices
+//   core: a symmetric bitmap of the edges among the last ranks, read by the
+//       counts instead of the lists of those vertices; its bits are set by the
+//       row kernels as they write the rows of those ranks
 //
 // The gather pass reads every adjacency entry once and looks up its rank, a
 // random 4-byte load from a 4n-byte table that stays in L2; that pass bounds
@@ -600,6 +601,28 @@ __device__ __forceinline__ uint32_t queue_key(int d, unsigned long long w)
     return (cls << 5) | (31u - quantise_work(w));
 }
 
+// The core: an adjacency bitmap of the ranks from lo on (rows of tw words, zeroed
+// beforehand).  lo = INT_MAX: none.
+struct Core {
+    uint32_t* bits;
+    int32_t lo, tw, n;
+};
+
+// Both bits of the edge of ranks r < y, if r is in the core (so is y, then).
+// The row kernels call it for every entry they store.  A kernel of its own over
+// the core's rows was another launch and another read of them: orientation 123 ->
+// 116 us at n = 1000, m = 10000, 218 -> 204 us on R-MAT of scale 17; where the core
+// has millions of edges the atomics bound both (Chung-Lu n = 3e5 297 -> 304 us, n =
+// 1e6 579 -> 581 us).  Tried: the words above the diagonal gathered in shared
+// memory and stored whole, 304 -> 295 and 581 -> 585 us, not worth it.
+__device__ __forceinline__ void core_edge(const Core& c, int32_t r, int32_t y)
+{
+    if (r < c.lo || y <= r || y >= c.n) return;
+    const int64_t x = r - c.lo, z = y - c.lo;
+    atomicOr(&c.bits[x * c.tw + (z >> 5)], 1u << (z & 31));
+    atomicOr(&c.bits[z * c.tw + (x >> 5)], 1u << (x & 31));
+}
+
 // Sort of one row of at most N entries held in shared memory, by one lane.
 template <int N>
 __device__ __forceinline__ void lane_sort(int32_t* s, int d)
@@ -631,7 +654,7 @@ __global__ void __launch_bounds__(kRowsThreads) k_rows(const int64_t* __restrict
                                                       const int32_t* __restrict__ tmp, int32_t n, int64_t m,
                                                       int32_t* __restrict__ adjp, uint32_t* __restrict__ qkey,
                                                       int32_t* __restrict__ widerows, int32_t* __restrict__ longrows,
-                                                      int64_t long_cap, Ctl* ctl)
+                                                      int64_t long_cap, Core core, Ctl* ctl)
 {
     __shared__ unsigned int h[256];
     __shared__ int32_t buf[kRowsThreads / 32][kRowsBuf];
@@ -699,7 +722,10 @@ __global__ void __launch_bounds__(kRowsThreads) k_rows(const int64_t* __restrict
             const int64_t rd0 = __shfl_sync(kFull, dst, lo);
             const bool rf = __shfl_sync(kFull, (int)fits, lo) != 0;
             const int fr = f - __shfl_sync(kFull, pre, lo);
-            if (f < T && rf) adjp[rd0 + fr] = sb[f];
+            if (f < T && rf) {
+                adjp[rd0 + fr] = sb[f];
+                core_edge(core, (int32_t)r0 + lo, sb[f]);
+            }
         }
         __syncwarp();
         const bool here = valid && d <= kRowsLane;
@@ -757,7 +783,7 @@ __device__ __forceinline__ void warp_reg_sort(int32_t (&x)[K], int lane)
 template <int K>
 __device__ __forceinline__ unsigned long long wide_row(const int32_t* __restrict__ src, int d,
                                                       const int32_t* __restrict__ dplus, int32_t* __restrict__ dst,
-                                                      bool fits, int lane)
+                                                      bool fits, int32_t r, const Core& core, int lane)
 {
     int32_t x[K];
 #pragma unroll
@@ -776,7 +802,10 @@ __device__ __forceinline__ unsigned long long wide_row(const int32_t* __restrict
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             const int j = k * 32 + lane;
-            if (j < d) dst[j] = x[k];
+            if (j < d) {
+                dst[j] = x[k];
+                core_edge(core, r, x[k]);
+            }
         }
     }
     return w;
@@ -792,7 +821,7 @@ __global__ void __launch_bounds__(kRowsThreads) k_rows_wide(const int64_t* __res
                                                            const int64_t* __restrict__ offp,
                                                            const int32_t* __restrict__ tmp, int64_t m,
                                                            int32_t* __restrict__ adjp, uint32_t* __restrict__ qkey,
-                                                           const int32_t* __restrict__ widerows, Ctl* ctl)
+                                                           const int32_t* __restrict__ widerows, Core core, Ctl* ctl)
 {
     __shared__ unsigned int h[256];
     for (int i = threadIdx.x; i < 256; i += kRowsThreads) h[i] = 0;
@@ -819,10 +848,10 @@ __global__ void __launch_bounds__(kRowsThreads) k_rows_wide(const int64_t* __res
             const int64_t dst = __shfl_sync(kFull, mdst, q);
             const bool fits = dst + d <= m;
             unsigned long long w;
-            if (d <= 64) w = wide_row<2>(src, d, dplus, adjp + dst, fits, lane);
-            else if (d <= 128) w = wide_row<4>(src, d, dplus, adjp + dst, fits, lane);
-            else if (d <= 256) w = wide_row<8>(src, d, dplus, adjp + dst, fits, lane);
-            else w = wide_row<16>(src, d, dplus, adjp + dst, fits, lane);
+            if (d <= 64) w = wide_row<2>(src, d, dplus, adjp + dst, fits, r, core, lane);
+            else if (d <= 128) w = wide_row<4>(src, d, dplus, adjp + dst, fits, r, core, lane);
+            else if (d <= 256) w = wide_row<8>(src, d, dplus, adjp + dst, fits, r, core, lane);
+            else w = wide_row<16>(src, d, dplus, adjp + dst, fits, r, core, lane);
             if (lane == 0) {
                 if (!fits) atomicOr(&ctl->st.err_input, 1);
                 const uint32_t key = queue_key(d, w);
@@ -848,7 +877,7 @@ __global__ void __launch_bounds__(kThreads) k_rows_long(const int64_t* __restric
                                                        const int64_t* __restrict__ offp, int32_t* __restrict__ tmp,
                                                        int64_t m, int32_t* __restrict__ adjp,
                                                        uint32_t* __restrict__ qkey, const int32_t* __restrict__ longrows,
-                                                       int64_t long_cap, Ctl* ctl)
+                                                       int64_t long_cap, Core core, Ctl* ctl)
 {
     __shared__ int32_t sb[kLongCap];
     __shared__ unsigned int s_row;
@@ -888,7 +917,10 @@ __global__ void __launch_bounds__(kThreads) k_rows_long(const int64_t* __restric
             }
         }
         if (fits)
-            for (int j = threadIdx.x; j < len; j += kThreads) adjp[dst + j] = s[j];
+            for (int j = threadIdx.x; j < len; j += kThreads) {
+                adjp[dst + j] = s[j];
+                core_edge(core, r, s[j]);
+            }
         if (threadIdx.x == 0) {
             if (!fits) atomicOr(&ctl->st.err_input, 1);
             const uint32_t key = queue_key(len, s_w);
@@ -939,25 +971,6 @@ int64_t core_ranks(int32_t n, int64_t m)
     int64_t t = std::min<int64_t>(n, kCoreMax);
     while (t > 128 && t * t > 32 * m) t -= std::max<int64_t>(1, t / 64);
     return m > 0 ? std::min<int64_t>((t + 127) & ~(int64_t)127, kCoreMax) : 0;
-}
-
-// Both bits of every edge inside the core, a warp per row of the core.  Bound:
-// atomics to the L2; Chung-Lu n = 1e6: 31 us of an orientation of 0.5 ms.
-__global__ void __launch_bounds__(kThreads) k_core(const int64_t* __restrict__ offp, const int32_t* __restrict__ adjp,
-                                                   int32_t n, int64_t m, int32_t lo, int tw, uint32_t* __restrict__ core)
-{
-    const int lane = threadIdx.x & 31;
-    const int nw = (int)(gridDim.x * blockDim.x) >> 5;
-    for (int32_t r = lo + (int32_t)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); r < n; r += nw) {
-        const int64_t e = min(offp[r + 1], m);  // (a CSR that was not symmetric: rows may be missing)
-        const int x = r - lo;
-        for (int64_t p = offp[r] + lane; p < e; p += 32) {
-            const int y = adjp[p] - lo;
-            if (y <= x || y >= n - lo) continue;
-            atomicOr(&core[(int64_t)x * tw + (y >> 5)], 1u << (y & 31));
-            atomicOr(&core[(int64_t)y * tw + (x >> 5)], 1u << (x & 31));
-        }
-    }
 }
 
 __global__ void k_zero_offset(int64_t* offp) { offp[0] = 0; }
@@ -1095,9 +1108,8 @@ kc_status orient(const int64_t* off_in, const int32_t* adj_in, int32_t n, int64_
     unsigned long long* sc_status = carve<unsigned long long>(sp, tiles);
     Ctl* ctl = carve<Ctl>(sp, 1);
     int* bad = carve<int>(sp, 1);
-    KC_CK(cudaMemsetAsync(sw_status, 0, (size_t)tiles * 256 * sweeps * sizeof(unsigned long long), s));
-    KC_CK(cudaMemsetAsync(sc_status, 0, (size_t)tiles * sizeof(unsigned long long), s));
-    KC_CK(cudaMemsetAsync(ctl, 0, sizeof(Ctl), s));
+    // the status words and ctl are neighbours: one fill
+    KC_CK(cudaMemsetAsync(sw_status, 0, (size_t)((char*)(ctl + 1) - (char*)sw_status), s));
 
     if (flags & KC_VALIDATE) {
         int64_t first = 0, last = 0;
@@ -1120,6 +1132,7 @@ kc_status orient(const int64_t* off_in, const int32_t* adj_in, int32_t n, int64_
         k_zero_offset<<<1, 1, 0, s>>>(g->offp);
         KC_LAUNCHED();
     } else {
+        const Core core{g->core, g->core_lo, g->core_tw, n};
         const int unit_grid = grid_for(((int64_t)n + 31) / 32 * 32, kThreads, sms * 8);
         // a1, a2: degrees, sort by degree (stable: ties in id order)
         k_degree<<<grid_for(n, kThreads, sms * 2), kThreads, 0, s>>>(off, n, kA, ctl);
@@ -1154,21 +1167,14 @@ kc_status orient(const int64_t* off_in, const int32_t* adj_in, int32_t n, int64_
                                                                              ctl);
         KC_LAUNCHED();
         k_rows<<<grid_for(((int64_t)n + 31) / 32 * 32, kRowsThreads, sms * 8), kRowsThreads, 0, s>>>(
-            off, g->perm, g->dplus, g->offp, tmp, n, m, g->adjp, kA, wide_rows, sort_rows, rows_cap, ctl);
+            off, g->perm, g->dplus, g->offp, tmp, n, m, g->adjp, kA, wide_rows, sort_rows, rows_cap, core, ctl);
         KC_LAUNCHED();
         k_rows_wide<<<sms * 16, kRowsThreads, 0, s>>>(off, g->perm, g->dplus, g->offp, tmp, m, g->adjp, kA, wide_rows,
-                                                     ctl);
+                                                     core, ctl);
         KC_LAUNCHED();
         k_rows_long<<<sms * 2, kThreads, 0, s>>>(off, g->perm, g->dplus, g->offp, tmp, m, g->adjp, kA, sort_rows,
-                                                 rows_cap, ctl);
+                                                 rows_cap, core, ctl);
         KC_LAUNCHED();
-
-        // adjacency bitmap of the last ranks, for the builds of G+(u)
-        if (g->core) {
-            k_core<<<grid_for((int64_t)(n - g->core_lo) * 32, kThreads, sms * 8), kThreads, 0, s>>>(
-                g->offp, g->adjp, n, m, g->core_lo, g->core_tw, g->core);
-            KC_LAUNCHED();
-        }
 
         // a5: owner queue (one pass on the 8-bit key; stable, so ties by rank)
         {
