@@ -56,6 +56,7 @@ typedef enum {
 /* flags */
 #define KC_DEVICE_PTRS 0x1u  /* array arguments are device pointers */
 #define KC_VALIDATE    0x2u  /* kc_orient / kc_count_csr: check the CSR first */
+#define KC_NO_CORE     0x4u  /* kc_orient: leave out the core bitmap (see kc_graph_info) */
 
 /* Largest k accepted by kc_count / kc_estimate. */
 #define KC_MAX_K 32
@@ -94,7 +95,10 @@ kc_status kc_build_csr(int32_t n, const int32_t* src, const int32_t* dst, int64_
  *   off, adj  the canonical CSR (arrays; host or, with KC_DEVICE_PTRS, device)
  *   n, m      vertices and undirected edges (adj has 2m entries); n >= 0
  *   flags     KC_DEVICE_PTRS, KC_VALIDATE (symmetry, sorted rows, no loops,
- *             no repeats; failures return KC_EINVAL)
+ *             no repeats; failures return KC_EINVAL), KC_NO_CORE (for callers
+ *             who export, list edges or hold many graphs more than they count:
+ *             less memory, up to 9 % less time here, same results everywhere,
+ *             slower counts at k >= 3)
  *   out       receives the new graph handle (NULL on failure)
  * Asynchronous on `stream` (without KC_VALIDATE): host inputs are copied
  * before the call returns; device inputs must stay unchanged until the
@@ -120,8 +124,11 @@ typedef struct {
     int32_t max_dplus;      /* max |Gamma+(u)|, at most 2 sqrt(m) (App. B, Thm I) */
     int64_t wedges;         /* sum over u of C(|Gamma+(u)|, 2): Map 2 pairs (App. B, Thm 1) */
     int64_t device_bytes;   /* device memory held by the handle: lists, offsets, per-vertex
-                               arrays, and an adjacency bitmap of the last ranks of the order
-                               (at most 16384 of them, and about 4 m bytes) */
+                               arrays, and the core bitmap: an adjacency bitmap of the last T
+                               ranks of the order, min(n, T) rows of T / 8 bytes.  T is a
+                               multiple of 128, at most 16384, and no larger than it takes to
+                               reach n, or sqrt(32 m) (4 m bytes), or 128.  Without KC_NO_CORE
+                               it is left out only where there is no memory for it. */
 } kc_graph_info;
 
 /* Statistics of an oriented graph (host struct).  Errors: KC_EINVAL. */

@@ -653,7 +653,7 @@ kc_status kc_count_csr(const int64_t* off, const int32_t* adj, int32_t n, int64_
                        uint64_t* total, uint64_t* per_vertex, uint64_t* per_owner, void* stream)
 {
     kc_graph* g = nullptr;
-    kc_status st = kc_orient(off, adj, n, m, flags, stream, &g);
+    kc_status st = kc_orient(off, adj, n, m, k <= 2 ? flags | KC_NO_CORE : flags, stream, &g);
     if (st != KC_OK) return st;
     st = kc_count(g, k, flags, total, per_vertex, per_owner, stream);
     if (st == KC_OK && (flags & KC_DEVICE_PTRS)) {

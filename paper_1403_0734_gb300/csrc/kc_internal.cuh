@@ -22,6 +22,7 @@ void set_cuda_error(cudaError_t e, const char* what);
         cudaError_t kc_e_ = (call);                                   \
         if (kc_e_ != cudaSuccess) {                                   \
             ::kc::set_cuda_error(kc_e_, #call);                       \
+            cudaGetLastError(); /* or the next launch reports it */   \
             return kc_e_ == cudaErrorMemoryAllocation ? KC_ENOMEM     \
                                                       : KC_ECUDA;     \
         }                                                             \

@@ -1011,8 +1011,10 @@ int num_sms()
     return sms;
 }
 
-kc_status orient(const int64_t* off_in, const int32_t* adj_in, int32_t n, int64_t m, unsigned flags,
-                 cudaStream_t s, kc_graph** out)
+namespace {
+
+kc_status orient_graph(const int64_t* off_in, const int32_t* adj_in, int32_t n, int64_t m, unsigned flags,
+                       bool with_core, cudaStream_t s, kc_graph** out)
 {
     *out = nullptr;
     if (n < 0 || m < 0 || (n == 0 && m != 0)) return KC_EINVAL;
@@ -1035,7 +1037,7 @@ kc_status orient(const int64_t* off_in, const int32_t* adj_in, int32_t n, int64_
 
     // resident arrays: one pool block
     {
-        const int64_t ranks = core_ranks(n, m);
+        const int64_t ranks = with_core ? core_ranks(n, m) : 0;
         if (ranks > 0) {
             g->core_lo = (int32_t)std::max<int64_t>(0, n - ranks);
             g->core_tw = (int32_t)(ranks / 32);
@@ -1052,10 +1054,7 @@ kc_status orient(const int64_t* off_in, const int32_t* adj_in, int32_t n, int64_
         g->queue = carve<int32_t>(p, nn);
         g->offp = carve<int64_t>(p, n1);
         g->adjp = carve<int32_t>(p, m);
-        if (ranks > 0) {
-            g->core = carve<uint32_t>(p, core_words);
-            KC_CK(cudaMemsetAsync(g->core, 0, (size_t)core_words * sizeof(uint32_t), s));
-        }
+        if (ranks > 0) g->core = carve<uint32_t>(p, core_words);
         g->bytes = (int64_t)bytes;
     }
     g->hstats = stats_slot_get();
@@ -1108,6 +1107,9 @@ kc_status orient(const int64_t* off_in, const int32_t* adj_in, int32_t n, int64_
     unsigned long long* sc_status = carve<unsigned long long>(sp, tiles);
     Ctl* ctl = carve<Ctl>(sp, 1);
     int* bad = carve<int>(sp, 1);
+    // (not before the last allocation: on failure the block is freed with nothing queued on it)
+    if (g->core)
+        KC_CK(cudaMemsetAsync(g->core, 0, (size_t)(n - g->core_lo) * g->core_tw * sizeof(uint32_t), s));
     // the status words and ctl are neighbours: one fill
     KC_CK(cudaMemsetAsync(sw_status, 0, (size_t)((char*)(ctl + 1) - (char*)sw_status), s));
 
@@ -1200,6 +1202,18 @@ kc_status orient(const int64_t* off_in, const int32_t* adj_in, int32_t n, int64_
     guard.keep = true;
     *out = g;
     return KC_OK;
+}
+
+}  // namespace
+
+// The core bitmap only saves time: a graph that does not fit with it goes without.
+kc_status orient(const int64_t* off_in, const int32_t* adj_in, int32_t n, int64_t m, unsigned flags,
+                 cudaStream_t s, kc_graph** out)
+{
+    const bool with_core = !(flags & KC_NO_CORE);
+    kc_status st = orient_graph(off_in, adj_in, n, m, flags, with_core, s, out);
+    if (st == KC_ENOMEM && with_core) st = orient_graph(off_in, adj_in, n, m, flags, false, s, out);
+    return st;
 }
 
 }  // namespace kc

@@ -19,6 +19,7 @@ LIB_PATH = os.path.join(_HERE, "libkc.so")
 KC_OK, KC_EINVAL, KC_ENOMEM, KC_EOVERFLOW, KC_ETIMEOUT, KC_ECUDA, KC_ENOTSUP, KC_ECANCELED = range(8)
 KC_DEVICE_PTRS = 0x1
 KC_VALIDATE = 0x2
+KC_NO_CORE = 0x4
 KC_MAX_K = 32
 KC_PARAM_SMEM_MAX_WORDS = 1
 KC_PARAM_LAUNCH_COUNT = 2
@@ -214,16 +215,18 @@ class Graph:
             pass
 
 
-def orient(off, adj, n: int | None = None, m: int | None = None, validate: bool = False, stream=None) -> Graph:
+def orient(off, adj, n: int | None = None, m: int | None = None, validate: bool = False, stream=None,
+           core: bool = True) -> Graph:
     """Round 1: degrees, (degree, id) order and Gamma+ lists on the device.
-    off/adj are numpy arrays (host) or torch CUDA tensors (device)."""
+    off/adj are numpy arrays (host) or torch CUDA tensors (device).
+    core=False leaves out the bitmap that only counts use (KC_NO_CORE)."""
     dev = _is_device(off)
     n = int(off.shape[0] - 1) if n is None else n
     m = int(adj.shape[0] // 2) if m is None else m
     if not dev:
         off = np.ascontiguousarray(off, dtype=np.int64)
         adj = np.ascontiguousarray(adj, dtype=np.int32)
-    flags = (KC_DEVICE_PTRS if dev else 0) | (KC_VALIDATE if validate else 0)
+    flags = (KC_DEVICE_PTRS if dev else 0) | (KC_VALIDATE if validate else 0) | (0 if core else KC_NO_CORE)
     h = _P()
     _check(_load().kc_orient(_ptr(off), _ptr(adj) if m > 0 else None, n, m, flags,
                              _stream_handle(stream), ctypes.byref(h)), "kc_orient")
