@@ -468,16 +468,18 @@ __device__ __forceinline__ void build_rows_small(const Ctx& c, const Gr& g, cons
             for (int w = h; w < W; ++w) up[h][w] = w == h ? val[h][w] & mask_above(lane) : val[h][w];
         }
     }
-    if (COL) {
-#pragma unroll 1
-        for (int i = 0; i < d - 1; ++i) {
-            const uint32_t ci = __shfl_sync(kFull, W == 1 || i < 32 ? col[0] : col[W - 1], i & 31);
+    if (COL) {  // (rows with an edge: random graph n = 5e5, m = 3e7, pairs at k = 4, 7.7 -> 6.7 ms)
 #pragma unroll
-            for (int w = 0; w < W; ++w) {
-                const uint32_t keep = __ballot_sync(kFull, sample_keep(c, ur, ci, col[w]));
-                if (lane == (i & 31)) {
-                    if (W == 1 || i < 32) up[0][w] &= keep;
-                    else up[W - 1][w] &= keep;
+        for (int h = 0; h < W; ++h) {
+            uint32_t rows = __ballot_sync(kFull, (up[h][0] | up[h][W - 1]) != 0u);
+#pragma unroll 1
+            for (; rows; rows &= rows - 1u) {
+                const int i = __ffs(rows) - 1;
+                const uint32_t ci = __shfl_sync(kFull, col[h], i);
+#pragma unroll
+                for (int w = 0; w < W; ++w) {
+                    const uint32_t keep = __ballot_sync(kFull, sample_keep(c, ur, ci, col[w]));
+                    if (lane == i) up[h][w] &= keep;
                 }
             }
         }

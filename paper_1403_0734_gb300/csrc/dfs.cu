@@ -750,8 +750,12 @@ __global__ void __launch_bounds__(256, 4) k_count_w2(Ctx cb, int take)
         cc::build_rows_small<2, COL>(cb, g, xs, d, cols, ur, sb, lane, rows);
         const unsigned long long u0 = ((unsigned long long)rows[0][1] << 32) | rows[0][0];  // upper rows of
         const unsigned long long u1 = ((unsigned long long)rows[1][1] << 32) | rows[1][0];  // lane, lane + 32
+        // elements that can be a clique's lowest inside G+(u); most owners of a
+        // graph without triangles to speak of have none, and nothing below runs
+        // (random graph n = 5e5, m = 3e7: k = 6 9.8 -> 9.5 ms)
+        const unsigned long long low = cvisit(~0ull, u0, u1, need - 1, lane);
         unsigned long long f0 = u0, f1 = u1;  // full rows (memberships, closing): add the transpose
-        if (PV || NEED == 4) {
+        if ((PV || NEED == 4) && low) {
             for (int j = 1; j < d; ++j) {
                 const unsigned long long colj = (unsigned long long)__ballot_sync(kFull, (u0 >> j) & 1ull) |
                                                 ((unsigned long long)__ballot_sync(kFull, (u1 >> j) & 1ull) << 32);
@@ -762,7 +766,8 @@ __global__ void __launch_bounds__(256, 4) k_count_w2(Ctx cb, int take)
         }
         unsigned long long a0 = 0, a1 = 0, wk = 0;
         unsigned long long tot = 0;
-        if constexpr (NEED == 0) {
+        if (low == 0ull) {
+        } else if constexpr (NEED == 0) {
             tot = cdfs<PV>(u0, u1, f0, f1, d, need, lane, a0, a1, cb.work ? &wk : nullptr);
         } else if constexpr (NEED == 3) {
             const int wid = threadIdx.x >> 5;
@@ -775,9 +780,7 @@ __global__ void __launch_bounds__(256, 4) k_count_w2(Ctx cb, int take)
             __syncwarp();
             const uint32_t share = 0x11111111u << (lane & 3);
             unsigned steps = 0;
-            // the lowest vertex of a 4-clique has three higher neighbours
-            const unsigned long long low = cvisit(~0ull, u0, u1, 3, lane);
-            for (int v0 = low ? 0 : d; v0 < d; v0 += 8) {
+            for (int v0 = 0; v0 < d; v0 += 8) {
                 const int v = v0 + (lane >> 2);
                 const uint2 X = v < d ? A[v] : make_uint2(0u, 0u);
                 const uint32_t take = PV || ((low >> (v & 63)) & 1ull) ? share : 0u;
@@ -839,10 +842,10 @@ __global__ void __launch_bounds__(256, 4) k_count_w2(Ctx cb, int take)
             ((uint4*)A)[lane + 32] = make_uint4((uint32_t)f1, (uint32_t)(f1 >> 32), 0u, 0u);
             if (PV) mine[lane] = mine[lane + 32] = 0ull;
             __syncwarp();
-            for (int e1 = 0; e1 < d; ++e1) {
+            for (unsigned long long left = low; left; left &= left - 1ull) {
+                const int e1 = __ffsll((long long)left) - 1;
                 const unsigned long long ue = crow(u0, u1, e1);
-                const int n = __popcll(ue);
-                if (n < NEED) continue;
+                const int n = __popcll(ue);  // at least NEED
                 cl::list_set<2, 32>(t, lane < 2 ? (uint32_t)(lane ? ue >> 32 : ue) : 0u, 2, lane, 0);
                 __syncwarp();
                 auto credit = [&](int j, uint32_t K) {
