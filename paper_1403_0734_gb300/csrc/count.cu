@@ -547,13 +547,32 @@ kc_status launch_slot_dfs(int slot, int Wh, const Ctx& c, uint32_t* heavy, int64
     return KC_OK;
 }
 
-kc_status launch_slot(int slot, int Wh, const Ctx& c, bool pv, bool col, uint32_t* heavy, int64_t heavy_words,
-                      Scratch* sc, const Plan* plan, cudaStream_t s)
+// Whether g's one-word owners are so small (at most 4.5 elements on average) that
+// at k = 3 the list search (k_tri_warp) is faster than rows in registers.  n = 1e6:
+// random graphs of m/n = 2, 4 0.237, 0.304 -> 0.149, 0.258 ms (5: 0.315 -> 0.337 with
+// the search's total sent per owner), triangular lattice 0.250 -> 0.201 ms, power-law
+// graphs of 3.6 and 5.3 elements on average 0.154 -> 0.138 and 0.410 -> 0.410 ms; n =
+// 2e4, m/n = 3 41 -> 36 us.  n = 1000: 34 -> 41 us, too few owners to hide the search's
+// longer chain of loads, hence kTriSmallMin.
+constexpr int64_t kTriSmallMin = 16384;
+
+bool tiny_owners(const kc_graph* g)
+{
+    const int64_t above = g->ge_small[33], items = g->ge_small[2] - above;
+    int64_t entries = 2 * items;
+    for (int t = 3; t <= 32; ++t) entries += g->ge_small[t] - above;
+    return 2 * entries <= 9 * items;
+}
+
+// tiny: tiny_owners of the graph (false for batches: one launch, many graphs).
+kc_status launch_slot(int slot, int Wh, const Ctx& c, bool pv, bool col, bool tiny, uint32_t* heavy,
+                      int64_t heavy_words, Scratch* sc, const Plan* plan, cudaStream_t s)
 {
     // No bitmaps for k = 3 but in registers: up to 64 elements the rows built
     // there beat the list search (Chung-Lu n = 1e6: 2.56 ms -> 0.33 + 0.92 ms).
     if (c.k == 3 && !col && tri_enabled()) {
-        if (slot_words(slot) == 1 || slot_words(slot) == 2)
+        const int W = slot_words(slot);
+        if ((W == 1 && !(tiny && c.nitems >= kTriSmallMin)) || W == 2)
             return pv ? launch_slot_dfs<true, false>(slot, Wh, c, heavy, heavy_words, sc, 1, s)
                       : launch_slot_dfs<false, false>(slot, Wh, c, heavy, heavy_words, sc, 1, s);
         return tri_launch_slot(slot, Wh, c, pv, s);
@@ -687,6 +706,7 @@ kc_status count_launch(const kc_graph* g, const CountArgs& a, unsigned long long
     if (a.nparts > 1) KC_TRY(graph_parts(g, a.nparts, s, &parts));
     const bool col = a.colours >= 2 || a.pair;  // one colour keeps every pair
     const int Wh = (g->max_dplus + 31) / 32;
+    const bool tiny = a.k == 3 && tiny_owners(g);
     for (int slot = 0; slot < kOwnerSlots; ++slot) {
         Ctx c = base;
         class_range(g, a.k, slot, &c.q0, &c.q1);
@@ -700,7 +720,7 @@ kc_status count_launch(const kc_graph* g, const CountArgs& a, unsigned long long
         }
         c.nitems = c.q1 - c.q0;
         c.cursor = cursors + slot;
-        KC_TRY(launch_slot(slot, Wh, c, a.per_vertex, col, heavy_scratch, heavy_words, a.sc, a.plan, s));
+        KC_TRY(launch_slot(slot, Wh, c, a.per_vertex, col, tiny, heavy_scratch, heavy_words, a.sc, a.plan, s));
     }
     return KC_OK;
 }
@@ -858,7 +878,7 @@ kc_status count_batch_run(const kc_graph* const* gs, int ng, const CountArgs& a,
         c.gpre = c.gq0 + ng;
         c.nitems = host_tables[(size_t)(slot * per + ng + ng)];
         c.cursor = cursors + slot;
-        KC_TRY(launch_slot(slot, Wh, c, false, col, heavy_scratch, heavy_words, a.sc, a.plan, s));
+        KC_TRY(launch_slot(slot, Wh, c, false, col, false, heavy_scratch, heavy_words, a.sc, a.plan, s));
     }
     return KC_OK;
 }
@@ -1002,7 +1022,7 @@ kc_status tune(const kc_graph* const* gs, int ng, int k, bool pv, cudaStream_t s
             for (int rep = 0; rep < 2; ++rep) {
                 KC_CK(cudaMemsetAsync(small, 0, (24 + 2 * (size_t)ng) * sizeof(unsigned long long), s));
                 KC_CK(cudaEventRecord(e0, s));
-                KC_TRY(launch_slot(slot, Wh, c, pv, false, heavy, hw, &sc, &pl, s));
+                KC_TRY(launch_slot(slot, Wh, c, pv, false, false, heavy, hw, &sc, &pl, s));
                 KC_CK(cudaEventRecord(e1, s));
                 KC_CK(cudaEventSynchronize(e1));
                 KC_CK(cudaEventElapsedTime(&ms, e0, e1));

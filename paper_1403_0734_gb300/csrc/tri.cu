@@ -6,7 +6,8 @@
 // (Sec. 4, the one- and two-round triangle algorithms it compares with).
 // Owners of more than 64 elements are counted here without building G+(u),
 // one CTA each with Gamma+(u) in shared memory (narrower ones take the one-warp
-// kernels of the bitmap path, whose rows are in registers anyway):
+// kernels of the bitmap path, whose rows are in registers anyway, but for many
+// owners of a few elements: k_tri_warp):
 //   * x_i in the core (a suffix of Gamma+(u)): its row of the core bitmap is
 //     tested at every later x_j, 32 at a time by a gather and a ballot;
 //   * other x_i: Gamma+(x_i) is streamed and every entry looked up in Gamma+(u)
@@ -35,6 +36,65 @@ using cc::Ctx;
 using cc::mask_below;
 
 constexpr int kSpanWords = 1024;                // direct table: spans up to 32768 ranks
+
+// Many owners of a few elements each, a warp per owner: Gamma+(u) in registers
+// (lane j holds x_j), every entry y of a 32-entry chunk of Gamma+(x_i) located by a
+// shuffle binary search.  Nothing is set up for an owner, where k_count_w1's hash
+// table and rows take some 200 instructions whatever the owner's size.  Single
+// graphs only (no batch tables).
+constexpr int kWarpItems = 4;  // owners a warp takes per cursor step
+
+template <bool PV>
+__global__ void __launch_bounds__(256) k_tri_warp(Ctx c)
+{
+    const int lane = threadIdx.x & 31;
+    unsigned long long sum = 0;
+    for (;;) {
+        unsigned long long pos0 = 0;
+        if (lane == 0) pos0 = atomicAdd(c.cursor, (unsigned long long)kWarpItems);
+        pos0 = __shfl_sync(kFull, pos0, 0);
+        if ((int64_t)pos0 >= c.nitems) break;
+        const int items = (int)min((int64_t)kWarpItems, c.nitems - (int64_t)pos0);
+        for (int it = 0; it < items; ++it) {
+            const int32_t r = c.queue[c.q0 + c.qoff + ((int64_t)pos0 + it) * c.qstride];
+            const int64_t b = c.offp[r];
+            const int d = (int)(c.offp[r + 1] - b);
+            const int32_t x = lane < d ? c.adjp[b + lane] : INT_MAX;
+            // offsets of every Gamma+(x_j) at once
+            const int64_t o0 = lane < d ? c.offp[x] : 0, o1 = lane < d ? c.offp[x + 1] : 0;
+            const int32_t maxL = __shfl_sync(kFull, x, d - 1);
+            uint32_t tot = 0, pvl = 0;
+            for (int i = 0; i < d - 1; ++i) {
+                const int64_t s0 = __shfl_sync(kFull, o0, i), s1 = __shfl_sync(kFull, o1, i);
+                uint32_t cnt = 0;
+                for (int64_t p0 = s0; p0 < s1; p0 += 32) {
+                    const int64_t p = p0 + lane;
+                    const int32_t y = p < s1 ? c.adjp[p] : INT_MAX;
+                    int lo = 0;
+#pragma unroll
+                    for (int step = 16; step > 0; step >>= 1) {
+                        const int32_t xx = __shfl_sync(kFull, x, lo + step - 1);
+                        if (xx < y) lo += step;
+                    }
+                    const int32_t xl = __shfl_sync(kFull, x, lo);
+                    const bool hit = y <= maxL && xl == y;
+                    cnt += (uint32_t)__popc(__ballot_sync(kFull, hit));
+                    if (PV) pvl += (__reduce_or_sync(kFull, hit ? (1u << lo) : 0u) >> lane) & 1u;
+                    if (__shfl_sync(kFull, y, 31) >= maxL) break;
+                }
+                tot += cnt;
+                if (PV && lane == i) pvl += cnt;
+            }
+            sum += tot;
+            if (lane == 0) {
+                if (c.po) c.po[r] = tot;
+                if (PV && tot) atomicAdd(&c.pv[r], (unsigned long long)tot);
+            }
+            if (PV && lane < d && pvl) atomicAdd(&c.pv[x], (unsigned long long)pvl);
+        }
+    }
+    if (lane == 0) add_total(c.total, sum);
+}
 
 // Shared layout (32-bit words): sL[D] ranks, sCnt[D] memberships (PV), the
 // span table's bitmap (kSpanWords) and 16-bit prefix counts (kSpanWords / 2).
@@ -161,11 +221,20 @@ kc_status set_tri(int64_t v)
 }
 
 // Owner slot `slot` (0: d+ above the shared-memory classes, 1..4: classes of
-// 32..4 words) of an exact k = 3 count.
+// 32..4 words, 6: one word) of an exact k = 3 count.
 kc_status tri_launch_slot(int slot, int Wh, const cc::Ctx& c, bool pv, cudaStream_t s)
 {
     if (c.nitems <= 0) return KC_OK;
     const int sms = num_sms();
+    if (slot == kOwnerSlots - 1) {
+        if (c.ng) return KC_ENOTSUP;
+        auto kern = pv ? k_tri_warp<true> : k_tri_warp<false>;
+        const int64_t warps = (c.nitems + kWarpItems - 1) / kWarpItems;
+        const int grid = (int)std::min<int64_t>((warps + 7) / 8, (int64_t)sms * cc::blocks_per_sm(kern, 256, 0));
+        kern<<<grid, 256, 0, s>>>(c);
+        KC_LAUNCHED();
+        return KC_OK;
+    }
     const int W = slot == 0 ? Wh : slot_words(slot);
     const int D = 32 * W;
     const size_t smem = (size_t)(D * (pv ? 2 : 1) + kSpanWords + kSpanWords / 2) * 4;

@@ -43,3 +43,19 @@ def check(kc, g, k):
 @pytest.mark.parametrize("k", [3, 4, 5, 6, 7])
 def test_sparse_two_word_owners(kc, n, per, cliques, size, k):
     check(kc, sparse(n, n * per, cliques, size, n + cliques), k)
+
+
+@pytest.mark.parametrize("n,per,cliques,size", [(30000, 2, 0, 0), (30000, 3, 400, 6), (40000, 4, 100, 20), (30000, 7, 0, 0),
+                                                (9000, 3, 50, 6)])
+def test_sparse_one_word_owners(kc, n, per, cliques, size):
+    # both sides of the rule at k = 3: on average 2.7..7 elements, more and fewer than 16384 owners
+    g = sparse(n, n * per, cliques, size, n + per)
+    check(kc, g, 3)
+    G = kc.orient(g.off, g.adj)
+    t, pv, po = kc.count(G, 3, per_vertex=True, per_owner=True)
+    parts = [kc.count_part(G, 3, p, 3, per_vertex=True, per_owner=True) for p in range(3)]
+    assert sum(p[0] for p in parts) == t
+    assert np.array_equal(sum(p[1] for p in parts), pv) and np.array_equal(sum(p[2] for p in parts), po)
+    got = np.sort(kc.list_cliques(G, 3), axis=1)
+    want = np.sort(oracle.list_cliques(g, 3), axis=1)
+    assert np.array_equal(got[np.lexsort(got.T)], want[np.lexsort(want.T)])
