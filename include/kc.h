@@ -395,8 +395,11 @@ void kc_batch_free(kc_batch* b);
  * For each class a plan names the Reduce 3 counter (KC_ALGO_DFS or
  * KC_ALGO_PIVOT, see KC_PARAM_ALGO) and, for the ordered search of classes
  * 1..5, the number of CTAs that share one owner (parts: 1 = no split; the
- * split owners' G+(u) is built once into a global tile).  A plan changes
- * speed only, never results.
+ * split owners' G+(u) is built once into a global tile).  Classes that are not
+ * searched ignore parts: k = 4 from 4 words on, k = 6 at 4 words; where the
+ * candidate sets of split owners are closed (k = 5 at 16 words, k = 6 at 8 and
+ * 16, see KC_PARAM_COMPLEMENT) every number above 1 means the same.  A plan
+ * changes speed only, never results.
  */
 typedef struct {
     int32_t k;           /* the k the plan is for */
@@ -411,8 +414,8 @@ typedef struct {
 /*
  * kc_tune -- measure, for every owner class of the ng graphs (one graph:
  * ng = 1), the candidate plans -- the ordered search with 1, 4 or 16 parts
- * per owner (4 and 16 only for classes of 8+ words at k >= 5) and the
- * pivoting counter -- on a sample of the class's heaviest owners (its first
+ * per owner (more than 1 only for classes of 4+ words at k >= 5, and only
+ * where it changes what runs) and the pivoting counter -- on a sample of the class's heaviest owners (its first
  * owners in queue order, at most 256), and return the fastest in `out`.  The
  * graphs are not changed (attach the plan with kc_set_tuning).  Runs
  * synchronously on `stream`.

@@ -54,6 +54,8 @@ kc_status set_count_algo(int64_t v)
 
 int64_t sct_heavy_words_w(int W, int k, int64_t nheavy);
 int parts_per_owner(int W, int k);
+bool parts_used(int W, int k);
+bool parts_close(int W, int k, int64_t items);
 kc_status sct_launch_slot(int slot, int Wh, const cc::Ctx& c, bool pv, bool col, uint32_t* heavy,
                           int64_t heavy_words, cudaStream_t s);
 bool dfs_reg_supported(int k);
@@ -532,8 +534,10 @@ kc_status launch_slot_dfs(int slot, int Wh, const Ctx& c, uint32_t* heavy, int64
     // at 4 words for k = 5 (both sides in quad.cu); on wider rows an edge's common
     // neighbours are too many to read each (dfs.cu and close.cu).
     // With memberships k = 5 reads whole rows, every 4-clique six times: the search
-    // is faster (Chung-Lu n = 1e6 21.0 -> 20.0 ms, R-MAT of scale 17 4.6 -> 3.2).
-    if ((k == 4 && W >= 4) || (k == 5 && W == 4 && !PV))
+    // is faster (Chung-Lu n = 1e6 21.0 -> 20.0 ms, R-MAT of scale 17 4.6 -> 3.2).  So
+    // is the search over several parts per owner where a plan asks for it: k = 5
+    // totals with 4 parts in every class, R-MAT of scale 15 0.92 -> 0.59 ms.
+    if ((k == 4 && W >= 4) || (k == 5 && W == 4 && !PV && (parts <= 1 || !sc)))
         return quad_launch(c, W, 32 * Wh, PV, COL, s);
     if (dfs_reg_supported(k)) return dfs_reg_launch(c, W, 32 * Wh, PV, COL, sc, parts, s);  // register-resident search
     const int NW = warps_for_width(W);
@@ -1006,9 +1010,13 @@ kc_status tune(const kc_graph* const* gs, int ng, int k, bool pv, cudaStream_t s
         const int W = slot_words(slot);
         std::vector<std::pair<int, int>> cand;  // (algo, parts)
         cand.push_back({KC_ALGO_DFS, 1});
-        if (slot >= 1 && slot < kOwnerSlots - 1 && W >= 4 && k >= 5 && dfs_reg_supported(k)) {
-            cand.push_back({KC_ALGO_DFS, 4});
-            cand.push_back({KC_ALGO_DFS, 16});
+        if (slot >= 1 && slot < kOwnerSlots - 1 && W >= 4 && k >= 5 && parts_used(W, k)) {
+            if (parts_close(W, k, nitems)) {
+                cand.push_back({KC_ALGO_DFS, parts_per_owner(W, k)});
+            } else {
+                cand.push_back({KC_ALGO_DFS, 4});
+                cand.push_back({KC_ALGO_DFS, 16});
+            }
         }
         cand.push_back({KC_ALGO_PIVOT, 1});
         float best = -1.0f;

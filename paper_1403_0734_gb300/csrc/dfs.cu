@@ -1301,11 +1301,22 @@ int parts_per_owner(int W, int k)
     return 1;
 }
 
+// Whether more than one part per owner changes what runs in the class of W words
+// at k: not in registers, not edge by edge (quad.cu, k = 4), not where a CTA closes
+// its owner's sets (close.cu, 4 words at k = 6).
+bool parts_used(int W, int k)
+{
+    return dfs_reg_supported(k) && W >= 2 && !(k == 4 && W >= 4) && !(k == 6 && W == 4 && g_complement);
+}
+
+// Whether all parts > 1 are the same there: the sets of split owners are closed.
+bool parts_close(int W, int k, int64_t items) { return g_complement && close_supported(W, k, items); }
+
 // Tile memory (32-bit words) a class of width W with `items` owners needs for
 // the split search at k (0: no split).
 int64_t dfs_tile_words(int W, int k, int64_t items, int parts)
 {
-    if ((parts > 0 ? parts : parts_per_owner(W, k)) <= 1 || items <= 0) return 0;
+    if (!parts_used(W, k) || (parts > 0 ? parts : parts_per_owner(W, k)) <= 1 || items <= 0) return 0;
     const int WM = W <= 16 ? W : 0;
     const int64_t per = 32LL * W * row_stride(W, WM);
     return per * items + (items + kCloseCursors + 3);  // tiles, then the task counters
@@ -1320,7 +1331,7 @@ kc_status dfs_reg_launch(const cc::Ctx& c, int W, int dmax, bool pv, bool col, S
     const int sms = num_sms();
     if (W == 4 && c.k == 6 && g_complement) return close_own_launch(c, col, s);
     int R = parts > 0 ? parts : parts_per_owner(W, c.k);
-    if (!sc) R = 1;
+    if (!sc || !parts_used(W, c.k)) R = 1;
     const int NW = W <= 4 ? 4 : 8;
     const int WM = W <= 16 ? W : 0;  // widest class keeps the generic last level
     // Totals at k >= 6 in the 4..16-word classes run on symmetric rows too:
@@ -1349,7 +1360,7 @@ kc_status dfs_reg_launch(const cc::Ctx& c, int W, int dmax, bool pv, bool col, S
         KC_LAUNCHED();
         return KC_OK;
     };
-    if (R > 1 && g_complement && close_supported(W, c.k, c.nitems)) {
+    if (R > 1 && parts_close(W, c.k, c.nitems)) {
         // tiles with the candidate-set sizes, then the sets of every size (close.cu)
         if (col) KC_TRY(W == 16 ? build_tiles(k_tile_build<true, true, 16>, ctr) : build_tiles(k_tile_build<true, true, 8>, ctr));
         else KC_TRY(W == 16 ? build_tiles(k_tile_build<true, false, 16>, ctr) : build_tiles(k_tile_build<true, false, 8>, ctr));
