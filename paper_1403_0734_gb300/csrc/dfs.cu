@@ -1360,7 +1360,14 @@ kc_status dfs_reg_launch(const cc::Ctx& c, int W, int dmax, bool pv, bool col, S
         KC_LAUNCHED();
         return KC_OK;
     };
-    if (R > 1 && parts_close(W, c.k, c.nitems)) {
+    // Rows thinned to half their pairs or so are the worst to close, neither they nor
+    // their complements are sparse.  Pair sampling at k = 5 is searched, closing against
+    // search: G(600, 0.7) p = 0.6, 0.8 1.38, 1.98 -> 0.91, 1.41 ms, Chung-Lu n = 1e6 13.1,
+    // 15.7 -> 10.6, 14.4 ms; at p = 0.95 2.4 -> 1.9 and 16.7 -> 18.2 ms.  (k = 6: closing is
+    // up to twice as fast on power-law graphs, and a third slower where p times the
+    // density of a dense graph is near one half.)
+    const bool thin = c.k == 5 && c.pair && c.pthr < 0xE666666666666666ull;  // p < 0.9
+    if (R > 1 && !thin && parts_close(W, c.k, c.nitems)) {
         // tiles with the candidate-set sizes, then the sets of every size (close.cu)
         if (col) KC_TRY(W == 16 ? build_tiles(k_tile_build<true, true, 16>, ctr) : build_tiles(k_tile_build<true, true, 8>, ctr));
         else KC_TRY(W == 16 ? build_tiles(k_tile_build<true, false, 16>, ctr) : build_tiles(k_tile_build<true, false, 8>, ctr));

@@ -59,3 +59,15 @@ def test_sparse_one_word_owners(kc, n, per, cliques, size):
     got = np.sort(kc.list_cliques(G, 3), axis=1)
     want = np.sort(oracle.list_cliques(g, 3), axis=1)
     assert np.array_equal(got[np.lexsort(got.T)], want[np.lexsort(want.T)])
+
+
+@pytest.mark.parametrize("p", [0.05, 0.4, 0.89, 0.91, 0.99])
+@pytest.mark.parametrize("k", [4, 5, 6])
+def test_pairs_in_wide_owners(kc, p, k):
+    # owners of 16 words, both sides of the rule at k = 5 (p = 0.9)
+    g = kcgen.from_edges(1100, np.random.default_rng(2).integers(1100, size=(200000, 2)), "wide")
+    G = kc.orient(g.off, g.adj)
+    assert 256 < G.max_dplus <= 512
+    s, _, spo = kc.estimate_pairs(G, k, p, 5, per_owner=True)
+    os_, _, ospo = oracle.estimate_pairs(g, k, p, 5, per_owner=True)
+    assert s == os_ and np.array_equal(spo, ospo)
