@@ -67,7 +67,8 @@ const char* kc_strerror(kc_status s);
 /* Text of the last CUDA error seen by this thread (static storage). */
 const char* kc_last_cuda_error(void);
 
-/* Library version, e.g. "kc 0.1 sm_103a". */
+/* Library version, e.g. "kc 0.2 sm_103a".  It changes with the kernels that plans
+ * (kc_tune) choose between. */
 const char* kc_version(void);
 
 /*

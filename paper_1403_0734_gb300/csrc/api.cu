@@ -198,7 +198,9 @@ const char* kc_strerror(kc_status s)
 
 const char* kc_last_cuda_error(void) { return kc::g_cuda_err; }
 
-const char* kc_version(void) { return "kc 0.1 sm_103a"; }
+// Cached plans are measured again under another version: a change of what a plan's
+// choices run, or of their speed, is a new one.
+const char* kc_version(void) { return "kc 0.2 sm_103a"; }
 
 kc_status kc_build_csr(int32_t n, const int32_t* src, const int32_t* dst, int64_t ne, int64_t* off,
                        int32_t* adj, int64_t* m_out)

@@ -447,7 +447,9 @@ def set_tuning(g: Graph, plan: dict | None):
 class TuningCache:
     """Plans cached in a JSON file, keyed by the graph's statistics (n, m,
     max |Gamma+|, wedges), k and the output mode, so a graph seen before (or
-    one with the same statistics) is not measured again."""
+    one with the same statistics) is not measured again.  A plan measured with
+    another version of the library ("lib", see kc_version; none in older files)
+    says nothing about this one's kernels: it is measured again and replaced."""
 
     def __init__(self, path: str):
         import json
@@ -466,8 +468,8 @@ class TuningCache:
         import json
         key = self.key(g, k, per_vertex)
         p = self.plans.get(key)
-        if p is None:
-            p = tune(g, k, per_vertex, stream)
+        if p is None or p.get("lib") != version():
+            p = dict(tune(g, k, per_vertex, stream), lib=version())
             self.plans[key] = p
             tmp = self.path + ".tmp"
             with open(tmp, "w") as f:
