@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(256) k_close_list(Ctx cb, Lists L, int chunks,
     for (int64_t it = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; it < cb.nitems * chunks; it += nw) {
         const int64_t oi = it / chunks;
         const int e = (int)(it - oi * chunks) * 32 + lane;
-        Ctx c;
+        cc::OwnerCtx c;
         int32_t r;
         if (!cc::resolve(cb, oi, c, r)) break;
         const int d = (int)(c.offp[r + 1] - c.offp[r]);
@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(cta_threads(WC), ctas_per_sm(WC)) k_close(Ctx 
         int deg = 0, size = 0;
         if (lane < have) {
             ent = L.entry(first + item + (unsigned)lane);
-            Ctx cl;
+            cc::OwnerCtx cl;
             int32_t own;
             cc::resolve(cb, ent >> 10, cl, own);
             at = cl.offp[own];
@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(cta_threads(WC), ctas_per_sm(WC)) k_close(Ctx 
             const uint32_t e = __shfl_sync(kFull, ent, i);
             const int64_t b = __shfl_sync(kFull, at, i);
             const int Wd = (__shfl_sync(kFull, deg, i) + 31) >> 5, n = __shfl_sync(kFull, size, i), e1 = (int)(e & 1023u);
-            Ctx c;
+            cc::OwnerCtx c;
             int32_t r;
             cc::resolve(cb, e >> 10, c, r);  // (always an item)
             const uint32_t* __restrict__ T = L.tiles + (int64_t)(e >> 10) * L.tile_words;
@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(kOwnWarps * 32, 8) k_close_own(Ctx cb)
     for (;;) {
         if (threadIdx.x == 0) s_item = (long long)atomicAdd(cb.cursor, 1ull);
         __syncthreads();
-        Ctx c;
+        cc::OwnerCtx c;
         int32_t r;
         if (!cc::resolve(cb, (int64_t)s_item, c, r)) break;
         const int64_t b = c.offp[r];

@@ -5,6 +5,7 @@
 #pragma once
 
 #include <climits>
+#include <type_traits>
 
 #include "kc_internal.cuh"
 
@@ -68,15 +69,28 @@ inline void set_graph(Ctx& c, const kc_graph* g)
     c.core_tw = g->core_tw;
 }
 
+// The context of one owner: a launch context with that owner's graph and total.
+// Only resolve fills it.  A variable that already holds a copy of the launch's
+// context, or takes it on another path, keeps the launch's offp after a resolve
+// compiled by nvcc 13.0 (32 of 32 lanes of a kernel that only compared the
+// pointers, with __restrict__ on Ctx's members and without); it is null in a batch.
+struct OwnerCtx : Ctx {
+    OwnerCtx() = default;
+    OwnerCtx(const Ctx&) = delete;
+    OwnerCtx(const OwnerCtx&) = delete;
+    OwnerCtx& operator=(const Ctx&) = delete;
+    OwnerCtx& operator=(const OwnerCtx&) = delete;
+};
+static_assert(!std::is_constructible<OwnerCtx, const Ctx&>::value && !std::is_assignable<OwnerCtx&, const Ctx&>::value &&
+                  !std::is_copy_constructible<OwnerCtx>::value && !std::is_copy_assignable<OwnerCtx>::value,
+              "an owner's context comes from resolve alone");
+
 // The owner (rank r) of class item `item`, with a context whose graph
-// pointers and total are that owner's graph's.  False past the last item.  c
-// must be a fresh variable: with one that already holds a copy of b, or that
-// takes b itself on another path, nvcc 13.0 leaves b's offp in it (seen by a
-// kernel that only compared the pointers).
-__device__ __forceinline__ bool resolve(const Ctx& b, int64_t item, Ctx& c, int32_t& r)
+// pointers and total are that owner's graph's.  False past the last item.
+__device__ __forceinline__ bool resolve(const Ctx& b, int64_t item, OwnerCtx& c, int32_t& r)
 {
     if (item >= b.nitems) return false;
-    c = b;
+    static_cast<Ctx&>(c) = b;
     if (b.ng == 0) {
         r = b.queue[b.q0 + b.qoff + item * b.qstride];
         return true;

@@ -1009,7 +1009,7 @@ __global__ void __launch_bounds__(256, 4) k_dfs_reg(Ctx cb, int W, int R, int cl
         if (threadIdx.x == 0) s_item = (long long)atomicAdd(cb.cursor, 1ull);
         __syncthreads();
         const int64_t oi = s_item / R;
-        Ctx c;
+        cc::OwnerCtx c;
         int32_t r;
         if (!cc::resolve(cb, oi, c, r)) break;
         const int64_t b = c.offp[r];
@@ -1222,7 +1222,7 @@ __global__ void __launch_bounds__(256) k_tile_build(Ctx cb, int W, uint32_t* til
         if (threadIdx.x == 0) s_item = (long long)atomicAdd(cb.cursor, 1ull);
         __syncthreads();
         const int64_t oi = s_item;
-        Ctx c;
+        cc::OwnerCtx c;
         int32_t r;
         if (!cc::resolve(cb, oi, c, r)) break;
         const int64_t b = c.offp[r];

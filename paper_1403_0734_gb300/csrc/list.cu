@@ -231,7 +231,7 @@ __global__ void __launch_bounds__(256) k_list(Ctx cb, int W, int levels, const u
         if (threadIdx.x == 0) s_item = (long long)atomicAdd(cb.cursor, 1ull);
         __syncthreads();
         const long long item = s_item;
-        Ctx c;
+        cc::OwnerCtx c;
         int32_t r;
         if (!cc::resolve(cb, (int64_t)item, c, r)) break;
         const int64_t b = c.offp[r];
@@ -449,7 +449,7 @@ __global__ void __launch_bounds__(256) k_list_reg(Ctx cb, const unsigned long lo
         if (threadIdx.x == 0) s_item = (long long)atomicAdd(cb.cursor, 1ull);
         __syncthreads();
         const long long item = s_item;
-        Ctx c;
+        cc::OwnerCtx c;
         int32_t r;
         if (!cc::resolve(cb, (int64_t)item, c, r)) break;
         const int64_t b = c.offp[r];
@@ -496,7 +496,7 @@ __global__ void __launch_bounds__(256) k_list_w1(Ctx cb, const unsigned long lon
         unsigned long long item = 0;
         if (lane == 0) item = atomicAdd(cb.cursor, 1ull);
         item = __shfl_sync(kFull, item, 0);
-        Ctx c;
+        cc::OwnerCtx c;
         int32_t r;
         if (!cc::resolve(cb, (int64_t)item, c, r)) break;
         const int64_t b = c.offp[r];
@@ -569,7 +569,7 @@ __global__ void k_list_small(Ctx cb, const unsigned long long* ooff, int32_t* ou
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t item = warp; item < cb.nitems; item += nwarps) {
-        Ctx c;
+        cc::OwnerCtx c;
         int32_t r;
         if (!cc::resolve(cb, item, c, r)) break;
         const int64_t o = (int64_t)ooff[item];

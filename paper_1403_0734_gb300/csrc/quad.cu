@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(WM <= 4 ? 128 : 256, WM <= 4 ? 8 : (WM <= 16 ?
     for (;;) {
         if (threadIdx.x == 0) s_item = (long long)atomicAdd(cb.cursor, 1ull);
         __syncthreads();
-        Ctx c;
+        cc::OwnerCtx c;
         int32_t r;
         if (!cc::resolve(cb, (int64_t)s_item, c, r)) break;
         const int64_t b = c.offp[r];

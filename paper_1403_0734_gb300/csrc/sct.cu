@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(256) k_sct_w1(Ctx cb)
         unsigned long long pos = 0;
         if (lane == 0) pos = atomicAdd(cb.cursor, 1ull);
         pos = __shfl_sync(kFull, pos, 0);
-        Ctx c;
+        cc::OwnerCtx c;
         int32_t r;
         if (!cc::resolve(cb, (int64_t)pos, c, r)) break;
         const int64_t b = c.offp[r];
@@ -273,7 +273,7 @@ __global__ void __launch_bounds__(256) k_sct_warp(Ctx cb, int W, uint32_t* gscra
         unsigned long long pos = 0;
         if (lane == 0) pos = atomicAdd(cb.cursor, 1ull);
         pos = __shfl_sync(kFull, pos, 0);
-        Ctx c;
+        cc::OwnerCtx c;
         int32_t r;
         if (!cc::resolve(cb, (int64_t)pos, c, r)) break;
         const int64_t b = c.offp[r];

@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(256) k_tri_cta(Ctx cb, int D)
             s_tot = 0ull;
         }
         __syncthreads();
-        Ctx c;
+        cc::OwnerCtx c;
         int32_t r;
         if (!cc::resolve(cb, (int64_t)s_item, c, r)) break;
         const int64_t b = c.offp[r];
