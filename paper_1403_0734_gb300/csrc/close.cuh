@@ -573,6 +573,8 @@ __device__ __forceinline__ unsigned long long close_set(const Team& t, int c, co
         if (K) credit(v, (uint32_t)K);
     }
     if (wk) {
+        // the edges of B, met once each by walk4 to find their triangles
+        if (NEED == 4 && tid == 0) *wk += (unsigned long long)(dense ? M : c * (c - 1) / 2 - M) * WC;
         *wk += (unsigned long long)steps * (unsigned)(WC * (NEED == 4 ? (dense ? 4 : 2) : 1));
 #pragma unroll 1
         for (int v = tid; v < c; v += NT) *wk += (unsigned long long)(Wd + (NEED == 4 && dense ? c * WC : 0));

@@ -138,3 +138,25 @@ def test_listing_order_and_alignment(kc, k):
     assert np.array_equal(got[0], got[1])
     a, b = np.sort(got[0], axis=1), np.sort(want, axis=1)
     assert np.array_equal(a[np.lexsort(a.T)], b[np.lexsort(b.T)])
+
+
+@pytest.mark.parametrize("pairs", [40, 65])
+def test_work_counter_counts_edges(kc, pairs):
+    # K_{2,2,...,2}: every candidate set's complement is a matching, edges without triangles.  Owners of more than
+    # 64 elements alone: less the work of the same graph's last 66 vertices.
+    def work(n):
+        G = kc.orient(*_csr(kcgen.complete_multipartite((2,) * n)))
+        kc.set_param(kc.KC_PARAM_WORK_COUNT, 1)
+        try:
+            t = kc.count(G, 6)[0]
+            return t, kc.get_param(kc.KC_PARAM_WORK_COUNT)
+        finally:
+            kc.set_param(kc.KC_PARAM_WORK_COUNT, 0)
+
+    want = 0
+    for half in range(33, pairs):          # two owners each, of 2 half elements
+        for c in range(4, 2 * half, 2):    # two sets each: rows squeezed, all rows met by each, the matching's edges
+            wc = 1 if c <= 32 else 4
+            want += 4 * (c * ((2 * half + 31) // 32 + c * wc) + c // 2 * wc)
+    (t, w), (_, last) = work(pairs), work(33)
+    assert t == comb(pairs, 6) * 64 and w - last == want
