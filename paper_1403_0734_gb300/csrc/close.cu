@@ -1,5 +1,6 @@
 // close.cu -- the counting kernels of the 4-, 8- and 16-word owner classes
-// that close candidate sets on compact copies (close.cuh).
+// that close candidate sets on compact copies (close.cuh); the 2-word class
+// closes its own in dfs.cu.
 //
 // 8 and 16 words (split classes): the owners' rows are in global tiles
 // (k_tile_build), the sets of all owners are listed by the row width of their
@@ -209,9 +210,10 @@ __host__ __device__ constexpr OwnLayout own_layout()
 // holds the vertices whose set is large enough: met one by one, empty sets took
 // as long as the rows' build (random graph n = 5e5, m = 3e7: whole count 9.5 ->
 // 8.3 ms).
-template <int NEED, bool COL>
+template <bool COL>
 __global__ void __launch_bounds__(kOwnWarps * 32, 8) k_close_own(Ctx cb)
 {
+    constexpr int NEED = 4;
     extern __shared__ __align__(16) char smem_close[];
     constexpr TeamLayout l = team_layout(4, 4, 1);
     constexpr OwnLayout o = own_layout();
@@ -373,7 +375,7 @@ kc_status close_own_launch(const Ctx& c, bool col, cudaStream_t s)
         KC_LAUNCHED();
         return KC_OK;
     };
-    return col ? go(k_close_own<4, true>) : go(k_close_own<4, false>);
+    return col ? go(k_close_own<true>) : go(k_close_own<false>);
 }
 
 }  // namespace kc

@@ -1,5 +1,5 @@
 // close.cuh -- candidate sets closed on a compact copy of their subgraph
-// (Reduce 3, Alg. 1; Sec. 3), for the 4-, 8- and 16-word owner classes.
+// (Reduce 3, Alg. 1; Sec. 3), for the 2-, 4-, 8- and 16-word owner classes.
 //
 // The ordered search of dfs.cu walks the chains x_i1 < x_i2 < ... until three
 // vertices are missing.  Here a candidate set C (the elements of G+(u) above
@@ -418,6 +418,7 @@ __device__ __forceinline__ unsigned long long close_set(const Team& t, int c, co
                                                         int Wd, int lane, int wid, unsigned long long* wk, Credit credit)
 {
     constexpr int NW = NT / 32;
+    static_assert(WC <= 16 && (NEED == 3 || NEED == 4), "32-bit sums hold up to 511 elements");
     const int wc = (c + 31) >> 5;
     const int tid = wid * 32 + lane;
     // 1. rows, and their degrees

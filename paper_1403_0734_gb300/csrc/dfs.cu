@@ -1,9 +1,9 @@
 // dfs.cu -- ordered depth-first counter (Reduce 3, Alg. 1; Sec. 3) for owners
-// whose G+(u) bitmap fits in shared memory (|Gamma+(u)| <= 1024), k <= 8: every
-// class at k >= 7, the 32-word class at k = 5 and 6, and what other rules leave
-// (quad.cu: k = 4, and k = 5 totals at 4 words; close.cu: k = 5 at 16 words and
-// k = 6 at 8 and 16 words in split tiles, k = 6 at 4 words; k_count_w2 below: two
-// words).
+// whose G+(u) bitmap fits in shared memory (|Gamma+(u)| <= 1024), k <= 8: the
+// classes of 4 and more words at k = 7 and 8, the 32-word class at k = 5 and 6, and
+// what other rules leave (quad.cu: k = 4, and k = 5 totals at 4 words unless split;
+// close.cu: k = 5 at 16 words and k = 6 at 8 and 16 words in split tiles, k = 6 at 4
+// words; k_count_w2 below: two words unless split; k_count_w1 in count.cu: one word).
 //
 // Same search as the generic kernel in count.cu -- chains x_i1 < x_i2 < ...
 // of G+(u) with candidate sets C_t = C_{t-1} & row(i_t), the last two levels
@@ -852,8 +852,8 @@ __global__ void __launch_bounds__(256, 4) k_count_w2(Ctx cb, int take)
                     if (PV) mine[t.pos[j]] += K;
                 };
                 const unsigned long long sub =
-                    n <= 32 ? cl::close_set<1, (NEED ? NEED : 4), 32>(t, n, A, kRS, 2, lane, 0, cb.work ? &wk : nullptr, credit)
-                            : cl::close_set<2, (NEED ? NEED : 4), 32>(t, n, A, kRS, 2, lane, 0, cb.work ? &wk : nullptr, credit);
+                    n <= 32 ? cl::close_set<1, 4, 32>(t, n, A, kRS, 2, lane, 0, cb.work ? &wk : nullptr, credit)
+                            : cl::close_set<2, 4, 32>(t, n, A, kRS, 2, lane, 0, cb.work ? &wk : nullptr, credit);
                 tot += sub;
                 if (PV && sub && lane == 0) mine[e1] += sub;
                 __syncwarp();

@@ -58,31 +58,10 @@ __device__ int set_pop(uint32_t* S, int& low, int W, int lane)
 // with WRITE, stores clique number pos + j for the j-th element.  Lanes
 // 0..t-1 hold the ids of the chain's levels in `chid`.
 template <bool WRITE>
-__device__ uint64_t leaves(const uint32_t* S, int low, int W, const int32_t* sL, int32_t uid, int32_t e1id, int t, int32_t chid, int32_t* out, int kk, int64_t pos,
-                           int64_t lim, int lane)
+__device__ uint64_t leaves(const uint32_t* S, int low, int W, const int32_t* sL, int32_t uid, int32_t e1id, int t,
+                           int32_t chid, int32_t* out, int kk, int64_t pos, int64_t lim, int lane)
 {
     uint64_t run = 0;
-    if (W <= 4) {  // few words: a lane per bit, no scan and no selection
-        const uint32_t lt = cc::mask_below(lane);
-        for (int w = low; w < W; ++w) {
-            const uint32_t v = S[w];
-            const int64_t row = pos + (int64_t)run + __popc(v & lt);
-            run += (uint64_t)__popc(v);
-            if (!WRITE || v == 0u) continue;
-            const bool ok = ((v >> lane) & 1u) && row < lim;  // rows past the run's buffer are never written
-            int32_t* o = out + row * kk;
-            for (int c = 0; c < t; ++c) {
-                const int32_t id = __shfl_sync(kFull, chid, c);
-                if (ok) o[2 + c] = id;
-            }
-            if (ok) {
-                o[0] = uid;
-                o[1] = e1id;
-                o[kk - 1] = sL[w * 32 + lane];
-            }
-        }
-        return run;
-    }
     for (int g0 = low; g0 < W; g0 += 32) {
         const int w = g0 + lane;
         const uint32_t v = w < W ? S[w] : 0u;

@@ -198,10 +198,8 @@ kc_status go(const Ctx& c, int D, cudaStream_t s)
 template <bool PV, bool COL>
 kc_status by_width(const Ctx& c, int W, int D, cudaStream_t s)
 {
-    if (c.k == 5) {
-        if constexpr (PV) return KC_ENOTSUP;
-        else return W == 4 ? go<PV, COL, 4, 5>(c, D, s) : KC_ENOTSUP;
-    }
+    if constexpr (!PV)
+        if (c.k == 5) return go<PV, COL, 4, 5>(c, D, s);
     switch (W) {
     case 4: return go<PV, COL, 4, 4>(c, D, s);
     case 8: return go<PV, COL, 8, 4>(c, D, s);
