@@ -1,7 +1,9 @@
 """Candidate sets closed on a compact copy of their subgraph (csrc/close.cu):
 every row width of the copy (1..16 words), both sides of the flip to the
 complement, against the oracle where it can enumerate the cliques, against
-closed forms, and against the ordered search (KC_PARAM_COMPLEMENT = 0)."""
+closed forms, and against the ordered search (KC_PARAM_COMPLEMENT = 0).
+
+Sets are closed at k = 5 and 6; the cases at k = 7 run the ordered search over the same graphs."""
 from math import comb
 
 import numpy as np
@@ -160,3 +162,66 @@ def test_work_counter_counts_edges(kc, pairs):
             want += 4 * (c * ((2 * half + 31) // 32 + c * wc) + c // 2 * wc)
     (t, w), (_, last) = work(pairs), work(33)
     assert t == comb(pairs, 6) * 64 and w - last == want
+
+
+def apex_over(parts):
+    """A vertex adjacent to all of a complete multipartite graph whose vertices have one pendant for each vertex of
+    their part: by degree the apex comes before them, so it is an owner of exactly sum(parts) elements."""
+    d = sum(parts)
+    label = np.repeat(np.arange(len(parts)), parts)
+    iu, ju = np.triu_indices(d, 1)
+    cross = label[iu] != label[ju]
+    size = np.array(parts)[label]
+    at = np.repeat(np.arange(d), size)
+    edges = [np.stack([iu[cross], ju[cross]], axis=1), np.stack([np.full(d, d), np.arange(d)], axis=1),
+             np.stack([at, d + 1 + np.arange(len(at))], axis=1)]
+    return kcgen.from_edges(d + 1 + len(at), np.concatenate(edges), f"apex_{d}"), label
+
+
+@pytest.mark.parametrize("k,d", [(k, d) for k in (5, 6) for d in (31, 32, 33, 63, 64, 65, 127, 128, 129, 255, 256, 257, 511, 512)]
+                         + [(5, 513), (4, 64), (4, 65), (4, 512), (4, 513)])
+def test_class_edges_multipartite(kc, k, d):
+    # eight unequal parts: cliques of every k, and complements that are cliques of different sizes
+    cut = [d * i * (i + 1) // 72 for i in range(9)]
+    parts = tuple(b - a for a, b in zip(cut, cut[1:]) if b > a)
+    assert sum(parts) == d and len(set(parts)) >= 5
+    g, label = apex_over(parts)
+    G = kc.orient(*_csr(g))
+    assert G.max_dplus == d
+    t, pv, po = counts(kc, G, k)
+    assert t == elementary((1,) + parts, k) > 0 and int(po[d]) == elementary(parts, k - 1)
+    for i, p in enumerate(parts):
+        rest = (1,) + parts[:i] + parts[i + 1:]
+        assert np.all(pv[:d][label == i] == elementary(rest, k - 1))
+    assert int(pv[d]) == elementary(parts, k - 1) and np.all(pv[d + 1:] == 0)
+
+
+@pytest.mark.parametrize("n,p", [(900, 0.4), (520, 0.55), (500, 0.7), (420, 0.9)])
+def test_close_matches_search_at_five(kc, n, p):
+    # 16-word owners at k = 5, their sets on both sides of half density
+    g = kcgen.random_small(n, p, 3 * n)
+    G = kc.orient(g.off, g.adj)
+    assert 257 <= G.max_dplus <= 512
+    got = counts(kc, G, 5)
+    kc.set_param(kc.KC_PARAM_COMPLEMENT, 0)
+    try:
+        want = counts(kc, G, 5)
+    finally:
+        kc.set_param(kc.KC_PARAM_COMPLEMENT, 1)
+    assert got[0] == want[0] and np.array_equal(got[1], want[1]) and np.array_equal(got[2], want[2])
+
+
+@pytest.mark.parametrize("maxw", [1, 2, 4])
+@pytest.mark.parametrize("k", [3, 4, 5])
+def test_listing_on_narrow_global_tiles(kc, maxw, k):
+    # owners of 2..8 words forced onto global tiles
+    g = kcgen.random_small(260, 0.35, 8)
+    G = kc.orient(*_csr(g))
+    want = oracle.list_cliques(g, k)
+    kc.set_param(kc.KC_PARAM_SMEM_MAX_WORDS, maxw)
+    try:
+        got = kc.list_cliques(G, k)
+    finally:
+        kc.set_param(kc.KC_PARAM_SMEM_MAX_WORDS, 32)
+    a, b = np.sort(got, axis=1), np.sort(want, axis=1)
+    assert np.array_equal(a[np.lexsort(a.T)], b[np.lexsort(b.T)])

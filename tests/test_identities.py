@@ -265,3 +265,60 @@ def test_k4_word_level_model(seed):
         assert [K[v] for v in sub] == b.tolist()
         checked += 1
     assert checked > 10
+
+
+# --- the sets closed on compact copies (csrc/close.cuh) -------------------
+
+def close_set_model(A, need):
+    """Cliques of `need` (3 or 4) vertices through every vertex of A as the kernel adds them up: the sparser of A and
+    its complement as B, sums credited edge by edge and triangle by triangle in twice or three times their value."""
+    c = A.shape[0]
+    N = [set(np.flatnonzero(A[v]).tolist()) for v in range(c)]
+    nb = [c - 1 - len(N[v]) for v in range(c)]
+    dense = 2 * sum(nb) <= c * (c - 1)
+    M = sum(nb) // 2
+    X = [set(range(c)) - {v} - N[v] for v in range(c)] if dense else N
+    acc, t, T = [0] * c, [0] * c, 0
+    edges = [(u, a) for u in range(c) for a in X[u] if a > u]
+    if need == 3:
+        for u, a in edges:
+            co = len(X[u] & X[a])
+            acc[u] += 2 * nb[a] - co if dense else co
+            acc[a] += 2 * nb[u] - co if dense else co
+        assert all(x % 2 == 0 for x in acc)
+        return [((c - 1 - nb[v]) * (c - 2 - nb[v]) // 2 - M if dense else 0) + acc[v] // 2 for v in range(c)]
+    if dense:
+        for v in range(c):
+            d, t2, s1, P2 = c - 1 - nb[v], 0, 0, 0
+            for a in range(c):
+                co = len(X[v] & X[a])
+                if a in X[v]:
+                    t2 += co
+                    s1 += nb[a]
+                else:  # v itself adds nothing: co = nb
+                    P2 += (nb[a] - co) * (nb[a] - co - 1)
+            t[v] = t2 // 2
+            acc[v] = -3 * (d * (d - 1) * (d - 2) // 6 - (M - s1 + t[v]) * (d - 2) + P2 // 2)
+        T = sum(t) // 3
+    for u, a in edges:
+        if dense:
+            acc[u] -= 3 * t[a]
+            acc[a] -= 3 * t[u]
+        for b in (b for b in X[u] & X[a] if b > a):
+            m = len(X[u] & X[a] & X[b])
+            for p, q, r in ((u, a, b), (a, u, b), (b, u, a)):
+                acc[p] += 3 * len(X[q] & X[r]) - m if dense else m
+    assert all(x % 3 == 0 for x in acc)
+    return [-T - acc[v] // 3 if dense else acc[v] // 3 for v in range(c)]
+
+
+@pytest.mark.parametrize("seed", range(6))
+def test_close_set_model(seed):
+    rng = np.random.default_rng(400 + seed)
+    for n in (3, 4, 7, 12, 18):
+        for p in (0.0, 0.2, 0.45, 0.5, 0.55, 0.8, 0.95, 1.0):
+            U = np.triu(rng.random((n, n)) < p, 1)
+            A = (U | U.T).astype(np.int64)
+            assert close_set_model(A, 3) == triangles_through(A).tolist(), (seed, n, p)
+            if n >= 4:
+                assert close_set_model(A, 4) == k4_through_brute(A).tolist(), (seed, n, p)
