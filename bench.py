@@ -47,19 +47,21 @@ METRIC = "k-cliques/sec and edges/sec at k=3..7 on 1 GB300; % HBM roofline; batc
 UNIT = "k-cliques/s"
 WORKLOAD = "chung_lu n=1e6 m~2e7 gamma=2.1 wmax=20000, exact k=3..6, per-vertex+per-owner"
 # the headline graph, and a reduced one of the same degree law for profiler
-# captures (its hubs still reach the 16-word class; a k = 6 count takes
-# ~0.3 s instead of ~1.1 s)
+# captures (its hubs still reach the 16-word class)
 GRAPHS = {"chunglu_1m": (1_000_000, 20_000_000, 2.1, 20000.0), "chunglu_300k": (300_000, 6_000_000, 2.1, 20000.0)}
 PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "roofline_traffic.json")
 # Word-operation peak of the counting kernels.  A word-op is one 32-bit AND
 # of a candidate-set word with a bitmap row word, its population count, and
-# the add of that count.  AND and add issue on the integer ALUs at 128 lanes
-# per SM per clock; the population count runs on the narrower unit that
-# serves POPC/FLO/BREV, at 16 lanes per SM per clock.  That unit is the
-# narrowest one every word-op needs, so the peak is 16 x SMs x SM clock
-# (the maximum SM clock of the measured peaks file).
+# the add of that count.  The population count runs on the narrowest unit
+# involved (POPC/FLO/BREV, 16 lanes per SM per clock), but the closing kernels
+# add words bitwise first: seven words take three population counts, the best
+# ratio of any row width (five words three, three words two).  So no call does
+# more than 16 x 7/3 word-ops per SM and clock, and the peak is that x SMs x
+# SM clock (the maximum SM clock of the measured peaks file).  What bounds the
+# kernels first is instruction issue; the ncu counters are in profiles/.
 POPC_LANES_PER_SM_CLK = 16
+WORDS_PER_POPC = 7 / 3
 # L2 random-gather rate measured on this GPU (4-byte loads at random
 # addresses of a 4 MB table, 8 warps per SM): the rate the orientation's one
 # gather pass over the adjacency is bound by.
@@ -561,7 +563,7 @@ def main():
     kmax_ms = statistics.mean(k_ms[kmax])
     clock_mhz = float(pk.get("sm_max_mhz", 2070.0))
     num_sms = torch.cuda.get_device_properties(local).multi_processor_count
-    peak_wops = POPC_LANES_PER_SM_CLK * num_sms * clock_mhz * 1e6 / 1e12  # Tword-op/s
+    peak_wops = POPC_LANES_PER_SM_CLK * WORDS_PER_POPC * num_sms * clock_mhz * 1e6 / 1e12  # Tword-op/s
     achieved = work / (kmax_ms * 1e-3) / 1e12
     traffic = None
     try:
@@ -573,7 +575,7 @@ def main():
         pass
     roofline = {"bound": "alu", "kernel": f"kc_count k={kmax} (counting kernels)", "achieved": achieved,
                 "peak": peak_wops, "unit": "Tword-op/s", "frac": achieved / peak_wops, "traffic": traffic,
-                "work_word_ops": work, "peak_kind": f"POPC lanes x SMs x {pk_kind} max SM clock",
+                "work_word_ops": work, "peak_kind": f"POPC lanes x 7/3 words per count x SMs x {pk_kind} max SM clock",
                 "plain_search_word_ops": work_plain,
                 "effective_frac": work_plain / (kmax_ms * 1e-3) / 1e12 / peak_wops}
     hbm = float(pk.get("hbm_gbs", 6800.0))

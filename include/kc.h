@@ -321,8 +321,8 @@ kc_status kc_count_batch(const kc_graph* const* gs, int ng, int k, unsigned flag
  *   KC_PARAM_LAUNCH_COUNT  read: kernels launched by this process so far;
  *       write 0 to reset.
  *   KC_PARAM_WORK_COUNT  write 1 (0) to turn on (off) work counting in the
- *       counting kernels; read: bitmap word-operations (a 32-bit AND plus
- *       population count) executed by the last synchronous kc_count /
+ *       counting kernels; read: bitmap word-operations (a 32-bit AND whose
+ *       bits are counted) executed by the last synchronous kc_count /
  *       kc_estimate on this process while counting was on.
  *   KC_PARAM_ALGO  the Reduce 3 counter used by kc_count / kc_estimate:
  *       KC_ALGO_DFS (default) enumerates ordered chains x_i1 < x_i2 < ... and
