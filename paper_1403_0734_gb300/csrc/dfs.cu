@@ -1331,6 +1331,16 @@ kc_status dfs_reg_launch(const cc::Ctx& c, int W, int dmax, bool pv, bool col, S
     const int sms = num_sms();
     if (W == 4 && c.k == 6 && g_complement) return close_own_launch(c, col, s);
     int R = parts > 0 ? parts : parts_per_owner(W, c.k);
+    // Rows thinned to half their pairs or so are the worst to close: neither they nor
+    // their complements are sparse.  Pair sampling at k = 5 is searched, over as many
+    // parts as it takes to fill the GPU.  Closing against 1, 4 and 16 parts, p = 0.6:
+    // G(600, 0.7), 239 owners, 1.38 and 1.70, 0.98, 0.91 ms; Chung-Lu n = 1e6, 3830 owners,
+    // 12.6 and 10.0, 9.7, 10.0 ms; random graph n = 1e5, m = 2e7, 36593 owners, 17.7 and
+    // 17.1, 20.6, 26.1 ms; at p = 0.95 Chung-Lu 16.7 and 18.2 ms over 16 parts.  (k = 6:
+    // closing is up to twice as fast on power-law graphs, and a third slower where p
+    // times the density of a dense graph is near one half.)
+    const bool thin = W == 16 && c.k == 5 && c.pair && c.pthr < 0xE666666666666666ull;  // p < 0.9
+    if (thin && parts <= 0) R = c.nitems >= 8192 ? 1 : (c.nitems >= 600 ? 4 : 16);
     if (!sc || !parts_used(W, c.k)) R = 1;
     const int NW = W <= 4 ? 4 : 8;
     const int WM = W <= 16 ? W : 0;  // widest class keeps the generic last level
@@ -1360,13 +1370,6 @@ kc_status dfs_reg_launch(const cc::Ctx& c, int W, int dmax, bool pv, bool col, S
         KC_LAUNCHED();
         return KC_OK;
     };
-    // Rows thinned to half their pairs or so are the worst to close, neither they nor
-    // their complements are sparse.  Pair sampling at k = 5 is searched, closing against
-    // search: G(600, 0.7) p = 0.6, 0.8 1.38, 1.98 -> 0.91, 1.41 ms, Chung-Lu n = 1e6 13.1,
-    // 15.7 -> 10.6, 14.4 ms; at p = 0.95 2.4 -> 1.9 and 16.7 -> 18.2 ms.  (k = 6: closing is
-    // up to twice as fast on power-law graphs, and a third slower where p times the
-    // density of a dense graph is near one half.)
-    const bool thin = c.k == 5 && c.pair && c.pthr < 0xE666666666666666ull;  // p < 0.9
     if (R > 1 && !thin && parts_close(W, c.k, c.nitems)) {
         // tiles with the candidate-set sizes, then the sets of every size (close.cu)
         if (col) KC_TRY(W == 16 ? build_tiles(k_tile_build<true, true, 16>, ctr) : build_tiles(k_tile_build<true, true, 8>, ctr));

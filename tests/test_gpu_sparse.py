@@ -71,3 +71,16 @@ def test_pairs_in_wide_owners(kc, p, k):
     s, _, spo = kc.estimate_pairs(G, k, p, 5, per_owner=True)
     os_, _, ospo = oracle.estimate_pairs(g, k, p, 5, per_owner=True)
     assert s == os_ and np.array_equal(spo, ospo)
+
+
+@pytest.mark.parametrize("n,m", [(1100, 200000), (3000, 600000), (24000, 7200000)])
+def test_pairs_over_parts(kc, n, m):
+    # some 150, 1000 and 11000 owners of 16 words: searched over 16, 4 parts and one
+    g = kcgen.from_edges(n, np.random.default_rng(3).integers(n, size=(m, 2)), "wide")
+    G = kc.orient(g.off, g.adj)
+    d = np.diff(kc.export(G)["off_plus"])
+    owners = int(((d > 256) & (d <= 512)).sum())
+    assert (owners >= 600) + (owners >= 8192) == [1100, 3000, 24000].index(n)
+    s, _, spo = kc.estimate_pairs(G, 5, 0.5, 5, per_owner=True)
+    os_, _, ospo = oracle.estimate_pairs(g, 5, 0.5, 5, per_owner=True)
+    assert s == os_ and np.array_equal(spo, ospo)
