@@ -844,7 +844,8 @@ __global__ void __launch_bounds__(256, 4) k_count_w2(Ctx cb, int take)
             __syncwarp();
             for (unsigned long long left = low; left; left &= left - 1ull) {
                 const int e1 = __ffsll((long long)left) - 1;
-                const unsigned long long ue = crow(u0, u1, e1);
+                const uint2 x = *(const uint2*)(A + kRS * e1);  // (u0, u1 would stay in registers)
+                const unsigned long long ue = (((unsigned long long)x.y << 32) | x.x) & (~1ull << e1);
                 const int n = __popcll(ue);  // at least NEED
                 cl::list_set<2, 32>(t, lane < 2 ? (uint32_t)(lane ? ue >> 32 : ue) : 0u, 2, lane, 0);
                 __syncwarp();
