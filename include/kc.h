@@ -98,7 +98,7 @@ kc_status kc_build_csr(int32_t n, const int32_t* src, const int32_t* dst, int64_
  *   flags     KC_DEVICE_PTRS, KC_VALIDATE (symmetry, sorted rows, no loops,
  *             no repeats; failures return KC_EINVAL), KC_NO_CORE (for callers
  *             who export, list edges or hold many graphs more than they count:
- *             less memory, up to 9 % less time here, same results everywhere,
+ *             less memory, up to 7 % less time here, same results everywhere,
  *             slower counts at k >= 3)
  *   out       receives the new graph handle (NULL on failure)
  * Asynchronous on `stream` (without KC_VALIDATE): host inputs are copied

@@ -609,12 +609,13 @@ struct Core {
 };
 
 // Both bits of the edge of ranks r < y, if r is in the core (so is y, then).
-// The row kernels call it for every entry they store.  A kernel of its own over
-// the core's rows was another launch and another read of them: orientation 123 ->
-// 116 us at n = 1000, m = 10000, 218 -> 204 us on R-MAT of scale 17; where the core
-// has millions of edges the atomics bound both (Chung-Lu n = 3e5 297 -> 304 us, n =
-// 1e6 579 -> 581 us).  Tried: the words above the diagonal gathered in shared
-// memory and stored whole, 304 -> 295 and 581 -> 585 us, not worth it.
+// The kernels of short and of very long rows call it for every entry they store;
+// the rows between are taken by the last of the row kernels, which has next to
+// nothing else to do.  A kernel of its own over the core's rows is another launch
+// (n = 1000, m = 10000: an orientation of 123 -> 117 us); bits set inside k_rows_wide
+// keep its few warps busy longer (Chung-Lu n = 3e5 307 -> 291 us, R-MAT of scale 20 608 -> 592 us).  Where the core has
+// millions of edges the atomics bound it all the same: Chung-Lu n = 1e6 579 -> 581 us,
+// 540 without a core.
 __device__ __forceinline__ void core_edge(const Core& c, int32_t r, int32_t y)
 {
     if (r < c.lo || y <= r || y >= c.n) return;
@@ -783,7 +784,7 @@ __device__ __forceinline__ void warp_reg_sort(int32_t (&x)[K], int lane)
 template <int K>
 __device__ __forceinline__ unsigned long long wide_row(const int32_t* __restrict__ src, int d,
                                                       const int32_t* __restrict__ dplus, int32_t* __restrict__ dst,
-                                                      bool fits, int32_t r, const Core& core, int lane)
+                                                      bool fits, int lane)
 {
     int32_t x[K];
 #pragma unroll
@@ -802,10 +803,7 @@ __device__ __forceinline__ unsigned long long wide_row(const int32_t* __restrict
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             const int j = k * 32 + lane;
-            if (j < d) {
-                dst[j] = x[k];
-                core_edge(core, r, x[k]);
-            }
+            if (j < d) dst[j] = x[k];
         }
     }
     return w;
@@ -821,7 +819,7 @@ __global__ void __launch_bounds__(kRowsThreads) k_rows_wide(const int64_t* __res
                                                            const int64_t* __restrict__ offp,
                                                            const int32_t* __restrict__ tmp, int64_t m,
                                                            int32_t* __restrict__ adjp, uint32_t* __restrict__ qkey,
-                                                           const int32_t* __restrict__ widerows, Core core, Ctl* ctl)
+                                                           const int32_t* __restrict__ widerows, Ctl* ctl)
 {
     __shared__ unsigned int h[256];
     for (int i = threadIdx.x; i < 256; i += kRowsThreads) h[i] = 0;
@@ -848,10 +846,10 @@ __global__ void __launch_bounds__(kRowsThreads) k_rows_wide(const int64_t* __res
             const int64_t dst = __shfl_sync(kFull, mdst, q);
             const bool fits = dst + d <= m;
             unsigned long long w;
-            if (d <= 64) w = wide_row<2>(src, d, dplus, adjp + dst, fits, r, core, lane);
-            else if (d <= 128) w = wide_row<4>(src, d, dplus, adjp + dst, fits, r, core, lane);
-            else if (d <= 256) w = wide_row<8>(src, d, dplus, adjp + dst, fits, r, core, lane);
-            else w = wide_row<16>(src, d, dplus, adjp + dst, fits, r, core, lane);
+            if (d <= 64) w = wide_row<2>(src, d, dplus, adjp + dst, fits, lane);
+            else if (d <= 128) w = wide_row<4>(src, d, dplus, adjp + dst, fits, lane);
+            else if (d <= 256) w = wide_row<8>(src, d, dplus, adjp + dst, fits, lane);
+            else w = wide_row<16>(src, d, dplus, adjp + dst, fits, lane);
             if (lane == 0) {
                 if (!fits) atomicOr(&ctl->st.err_input, 1);
                 const uint32_t key = queue_key(d, w);
@@ -871,13 +869,15 @@ constexpr int kLongCap = 8192;  // kept entries a CTA sorts in shared memory
 
 // Rows of more than kRowsWarp entries: one CTA per row sorts it (in shared
 // memory up to kLongCap entries, else in place in tmp), copies it, and sets
-// its queue key.
+// its queue key.  Then the core's bits of the rows k_rows_wide has written, a warp
+// per row.
 __global__ void __launch_bounds__(kThreads) k_rows_long(const int64_t* __restrict__ off, const int32_t* __restrict__ perm,
                                                        const int32_t* __restrict__ dplus,
                                                        const int64_t* __restrict__ offp, int32_t* __restrict__ tmp,
                                                        int64_t m, int32_t* __restrict__ adjp,
                                                        uint32_t* __restrict__ qkey, const int32_t* __restrict__ longrows,
-                                                       int64_t long_cap, Core core, Ctl* ctl)
+                                                       int64_t long_cap, const int32_t* __restrict__ widerows,
+                                                       Core core, Ctl* ctl)
 {
     __shared__ int32_t sb[kLongCap];
     __shared__ unsigned int s_row;
@@ -928,6 +928,17 @@ __global__ void __launch_bounds__(kThreads) k_rows_long(const int64_t* __restric
             atomicAdd(&ctl->qhist[0][key], 1u);
         }
         __syncthreads();
+    }
+    if (core.lo >= core.n) return;
+    const unsigned int nwide = ctl->nwide_rows;
+    const int lane = threadIdx.x & 31;
+    for (unsigned int i = (blockIdx.x * kThreads + threadIdx.x) >> 5; i < nwide; i += gridDim.x * (kThreads / 32)) {
+        const int32_t r = widerows[i];
+        if (r < core.lo) continue;
+        const int d = dplus[r];
+        const int64_t b = offp[r];
+        if (b + d > m) continue;
+        for (int j = lane; j < d; j += 32) core_edge(core, r, adjp[b + j]);
     }
 }
 
@@ -1172,10 +1183,12 @@ kc_status orient_graph(const int64_t* off_in, const int32_t* adj_in, int32_t n, 
             off, g->perm, g->dplus, g->offp, tmp, n, m, g->adjp, kA, wide_rows, sort_rows, rows_cap, core, ctl);
         KC_LAUNCHED();
         k_rows_wide<<<sms * 16, kRowsThreads, 0, s>>>(off, g->perm, g->dplus, g->offp, tmp, m, g->adjp, kA, wide_rows,
-                                                     core, ctl);
+                                                     ctl);
         KC_LAUNCHED();
-        k_rows_long<<<sms * 2, kThreads, 0, s>>>(off, g->perm, g->dplus, g->offp, tmp, m, g->adjp, kA, sort_rows,
-                                                 rows_cap, core, ctl);
+        // CTAs for a warp per row of the core, at most as many as fit
+        const int long_grid = std::max(sms * 2, grid_for((int64_t)(g->core ? n - g->core_lo : 0) * 32, kThreads, sms * 6));
+        k_rows_long<<<long_grid, kThreads, 0, s>>>(off, g->perm, g->dplus, g->offp, tmp, m, g->adjp, kA, sort_rows,
+                                                   rows_cap, wide_rows, core, ctl);
         KC_LAUNCHED();
 
         // a5: owner queue (one pass on the 8-bit key; stable, so ties by rank)
