@@ -18,7 +18,7 @@
 //       entries Round 2 reads for u), descending; ties by rank.
 //   core: a symmetric bitmap of the edges among the last ranks, read by the
 //       counts instead of the lists of those vertices; its bits are set by the
-//       row kernels as they write the rows of those ranks
+//       row kernels
 //
 // The gather pass reads every adjacency entry once and looks up its rank, a
 // random 4-byte load from a 4n-byte table that stays in L2; that pass bounds
@@ -612,10 +612,10 @@ struct Core {
 // The kernels of short and of very long rows call it for every entry they store;
 // the rows between are taken by the last of the row kernels, which has next to
 // nothing else to do.  A kernel of its own over the core's rows is another launch
-// (n = 1000, m = 10000: an orientation of 123 -> 117 us); bits set inside k_rows_wide
-// keep its few warps busy longer (Chung-Lu n = 3e5 307 -> 291 us, R-MAT of scale 20 608 -> 592 us).  Where the core has
-// millions of edges the atomics bound it all the same: Chung-Lu n = 1e6 579 -> 581 us,
-// 540 without a core.
+// (n = 1000, m = 10000: an orientation of 123 -> 117 us); bits set inside
+// k_rows_wide keep its few warps busy longer (Chung-Lu n = 3e5 307 -> 291 us, R-MAT
+// of scale 20 608 -> 592 us).  Where the core has millions of edges the atomics
+// bound it all the same: Chung-Lu n = 1e6 579 -> 581 us, 540 without a core.
 __device__ __forceinline__ void core_edge(const Core& c, int32_t r, int32_t y)
 {
     if (r < c.lo || y <= r || y >= c.n) return;
