@@ -588,6 +588,7 @@ def main():
     orient_roof["frac"] = orient_roof["achieved"] / hbm
     orient_roof["frac_of_gather_bound"] = orient_roof["l2_gather_bound_ms"] / om
     # Round 2 (the build of every G+(u)): its input bytes over the k = 3, 4 calls
+    # (an effective rate: the core's lists are not read any more, so it can pass HBM's)
     build_roof = {"bound": "hbm", "peak": hbm, "unit": "GB/s",
                   "per_k": {str(k): {"round2_bytes": r2[k], "ms": statistics.mean(k_ms[k]),
                                      "achieved": r2[k] / (statistics.mean(k_ms[k]) * 1e-3) / 1e9,
