@@ -348,7 +348,8 @@ kc_status kc_count_batch(const kc_graph* const* gs, int ng, int k, unsigned flag
  *       stops one level earlier in the 2- to 16-word classes (8 and 16 words:
  *       where the rows are in split tiles), k = 5 in the 16-word class: a candidate set
  *       that needs three or four vertices is closed on a compact copy of its
- *       subgraph, through the complement when that is the sparser side.  0:
+ *       subgraph, through the complement when that is the sparser side (not
+ *       where density and sampling leave rows about half full).  0:
  *       every such set is closed on its edges (one row read per neighbour) and
  *       totals keep upper-triangular rows.
  * kc_set_param returns KC_EINVAL for an unknown knob or a value out of range.

@@ -55,7 +55,7 @@ kc_status set_count_algo(int64_t v)
 int64_t sct_heavy_words_w(int W, int k, int64_t nheavy);
 int parts_per_owner(int W, int k);
 bool parts_used(int W, int k);
-bool parts_close(int W, int k, int64_t items);
+bool sets_closed(const cc::Ctx& c, int W, int64_t items, bool pv);
 kc_status sct_launch_slot(int slot, int Wh, const cc::Ctx& c, bool pv, bool col, uint32_t* heavy,
                           int64_t heavy_words, cudaStream_t s);
 bool dfs_reg_supported(int k);
@@ -620,6 +620,7 @@ Ctx base_ctx(const CountArgs& a)
     c.po = a.po;
     c.cursor = nullptr;
     c.work = a.work;
+    c.density = 0.0f;
     return c;
 }
 
@@ -865,6 +866,24 @@ void batch_tables(const kc_graph* const* gs, int ng, int k, std::vector<int64_t>
     }
 }
 
+namespace {
+
+// Of a batch: the largest density of its graphs with owners of 16 words, where all
+// of those are dense (sets_closed); else 0.
+float batch_density(const kc_graph* const* gs, int ng)
+{
+    float lo = 2.0f, hi = 0.0f;
+    for (int g = 0; g < ng; ++g)
+        if (gs[g]->max_dplus > 256) {
+            const float d = cc::density_of(gs[g]);
+            lo = std::min(lo, d);
+            hi = std::max(hi, d);
+        }
+    return lo >= 1.0f / 16 ? hi : 0.0f;
+}
+
+}  // namespace
+
 kc_status count_batch_run(const kc_graph* const* gs, int ng, const CountArgs& a, const void* descs,
                           const int64_t* tables, const std::vector<int64_t>& host_tables, unsigned long long* cursors,
                           uint32_t* heavy_scratch, int64_t heavy_words, cudaStream_t s)
@@ -872,6 +891,7 @@ kc_status count_batch_run(const kc_graph* const* gs, int ng, const CountArgs& a,
     Ctx base = base_ctx(a);
     base.gd = (const cc::GraphDesc*)descs;
     base.ng = ng;
+    base.density = batch_density(gs, ng);
     const bool col = a.colours >= 2 || a.pair;
     int Wh = 1;
     for (int g = 0; g < ng; ++g) Wh = std::max(Wh, (gs[g]->max_dplus + 31) / 32);
@@ -979,6 +999,7 @@ kc_status tune(const kc_graph* const* gs, int ng, int k, bool pv, cudaStream_t s
         KC_CK(cudaStreamSynchronize(s));
         base.gd = dd;
         base.ng = ng;
+        base.density = batch_density(gs, ng);
         base.total = small + 16;
     }
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -1011,7 +1032,7 @@ kc_status tune(const kc_graph* const* gs, int ng, int k, bool pv, cudaStream_t s
         std::vector<std::pair<int, int>> cand;  // (algo, parts)
         cand.push_back({KC_ALGO_DFS, 1});
         if (slot >= 1 && slot < kOwnerSlots - 1 && W >= 4 && k >= 5 && parts_used(W, k)) {
-            if (parts_close(W, k, nitems)) {
+            if (sets_closed(c, W, nitems, pv)) {
                 cand.push_back({KC_ALGO_DFS, parts_per_owner(W, k)});
             } else {
                 cand.push_back({KC_ALGO_DFS, 4});

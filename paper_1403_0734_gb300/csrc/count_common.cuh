@@ -56,7 +56,13 @@ struct Ctx {
     unsigned long long* po;
     unsigned long long* cursor;
     unsigned long long* work;  // nullable: bitmap word-operations executed
+    float density;             // for the host's dispatch: edges / pairs of vertices (density_of)
 };
+
+inline float density_of(const kc_graph* g)
+{
+    return g->n > 1 ? (float)(2.0 * (double)g->m / ((double)g->n * (g->n - 1.0))) : 0.0f;
+}
 
 inline void set_graph(Ctx& c, const kc_graph* g)
 {
@@ -67,6 +73,7 @@ inline void set_graph(Ctx& c, const kc_graph* g)
     c.core = g->core;
     c.core_lo = g->core_lo;
     c.core_tw = g->core_tw;
+    c.density = density_of(g);
 }
 
 // The context of one owner: a launch context with that owner's graph and total.

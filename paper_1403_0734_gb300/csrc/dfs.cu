@@ -1310,8 +1310,29 @@ bool parts_used(int W, int k)
     return dfs_reg_supported(k) && W >= 2 && !(k == 4 && W >= 4) && !(k == 6 && W == 4 && g_complement);
 }
 
-// Whether all parts > 1 are the same there: the sets of split owners are closed.
-bool parts_close(int W, int k, int64_t items) { return g_complement && close_supported(W, k, items); }
+// Whether the sets of the class's split owners are closed (all parts > 1 are the
+// same then), not searched.  Rows about half full are the worst to close: neither
+// they nor their complements are sparse.  A graph that is itself dense says how full
+// they are (in a sparse graph the wide owners are hubs, whose rows may be anything,
+// mostly full: closed); pair sampling thins them.  Closing against search:
+//   k = 5, no memberships, graphs of density 1/16 to 0.8: G(900, 0.5) 2.45 -> 1.62 ms,
+//   G(600, 0.7) 2.29 -> 1.97 ms, G(1500, 0.4) 12.2 -> 10.9 ms; G(520, 0.9) 2.8 -> 4.0
+//   ms, Chung-Lu n = 1e6 13.6 -> 17.0 ms.  With memberships closing wins, G(600, 0.7) 3.0
+//   against 4.0 ms.
+//   k = 5, pairs at p = 0.6: Chung-Lu n = 1e6 12.6 -> 9.7 ms, G(600, 0.7) 1.38 -> 0.91
+//   ms; at p = 0.95 Chung-Lu 16.7 -> 18.2 ms.
+//   k = 6, pairs of dense graphs, p times density: 0.42, 0.54, 0.58 G(600, 0.7) 9.8 -> 7.8
+//   ms, G(520, 0.9) 34.3 -> 23.0 ms, K_{7,9,11,13 x 12} 37.4 -> 29.9 ms; 0.30 G(600, 0.5)
+//   1.24 -> 1.71 ms, 0.67 G(600, 0.7) 20.5 -> 38.2 ms.
+bool sets_closed(const cc::Ctx& c, int W, int64_t items, bool pv)
+{
+    if (!g_complement || !close_supported(W, c.k, items)) return false;
+    const double kept = c.pair ? (double)c.pthr * 0x1p-64 : 1.0;
+    const bool dense = c.density >= 1.0f / 16;
+    if (c.k == 5) return pv || !(kept < 0.9 || (dense && c.density <= 0.8f));
+    const double full = kept * c.density;
+    return !(c.pair && dense && full > 0.41 && full < 0.62);
+}
 
 // Tile memory (32-bit words) a class of width W with `items` owners needs for
 // the split search at k (0: no split).
@@ -1332,16 +1353,13 @@ kc_status dfs_reg_launch(const cc::Ctx& c, int W, int dmax, bool pv, bool col, S
     const int sms = num_sms();
     if (W == 4 && c.k == 6 && g_complement) return close_own_launch(c, col, s);
     int R = parts > 0 ? parts : parts_per_owner(W, c.k);
-    // Rows thinned to half their pairs or so are the worst to close: neither they nor
-    // their complements are sparse.  Pair sampling at k = 5 is searched, over as many
-    // parts as it takes to fill the GPU.  Closing against 1, 4 and 16 parts, p = 0.6:
-    // G(600, 0.7), 239 owners, 1.38 and 1.70, 0.98, 0.91 ms; Chung-Lu n = 1e6, 3830 owners,
-    // 12.6 and 10.0, 9.7, 10.0 ms; random graph n = 1e5, m = 2e7, 36593 owners, 17.7 and
-    // 17.1, 20.6, 26.1 ms; at p = 0.95 Chung-Lu 16.7 and 18.2 ms over 16 parts.  (k = 6:
-    // closing is up to twice as fast on power-law graphs, and a third slower where p
-    // times the density of a dense graph is near one half.)
-    const bool thin = W == 16 && c.k == 5 && c.pair && c.pthr < 0xE666666666666666ull;  // p < 0.9
-    if (thin && parts <= 0) R = c.nitems >= 8192 ? 1 : (c.nitems >= 600 ? 4 : 16);
+    // The search that takes the place of closing runs over as many parts as it takes
+    // to fill the GPU.  Pairs at k = 5, p = 0.6, 1, 4 and 16 parts: 239 owners of G(600, 0.7)
+    // 1.70, 0.98, 0.91 ms; 3830 of Chung-Lu n = 1e6 10.0, 9.7, 10.0 ms; 36593 of a random
+    // graph n = 1e5, m = 2e7 17.1, 20.6, 26.1 ms (closed 17.7).
+    const bool closed = sets_closed(c, W, c.nitems, pv);
+    if (!closed && parts <= 0 && g_complement && close_supported(W, c.k, c.nitems))
+        R = c.nitems >= 8192 ? 1 : (c.nitems >= 600 ? std::min(R, 4) : R);
     if (!sc || !parts_used(W, c.k)) R = 1;
     const int NW = W <= 4 ? 4 : 8;
     const int WM = W <= 16 ? W : 0;  // widest class keeps the generic last level
@@ -1371,7 +1389,7 @@ kc_status dfs_reg_launch(const cc::Ctx& c, int W, int dmax, bool pv, bool col, S
         KC_LAUNCHED();
         return KC_OK;
     };
-    if (R > 1 && !thin && parts_close(W, c.k, c.nitems)) {
+    if (R > 1 && closed) {
         // tiles with the candidate-set sizes, then the sets of every size (close.cu)
         if (col) KC_TRY(W == 16 ? build_tiles(k_tile_build<true, true, 16>, ctr) : build_tiles(k_tile_build<true, true, 8>, ctr));
         else KC_TRY(W == 16 ? build_tiles(k_tile_build<true, false, 16>, ctr) : build_tiles(k_tile_build<true, false, 8>, ctr));

@@ -67,7 +67,8 @@ def test_launches_of_parts(kc, graph, k, slot, used, pv):
 def test_tuner_times_what_differs(kc, graph, k, pv):
     p = kc.tune(graph[1], k, per_vertex=pv)
     assert p["parts"][W4] in ((1,) if k == 6 else (1, 4, 16))
-    assert p["parts"][W16] in (1, 16)
+    # (a graph of density 0.7: totals at k = 5 are searched in the 16-word class, the others closed)
+    assert p["parts"][W16] in ((1, 4, 16) if k == 5 and not pv else (1, 16))
     assert p["parts"][W8] in ((1, 4) if k == 6 else (1, 4, 16))
 
 

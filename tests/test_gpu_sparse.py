@@ -84,3 +84,35 @@ def test_pairs_over_parts(kc, n, m):
     s, _, spo = kc.estimate_pairs(G, 5, 0.5, 5, per_owner=True)
     os_, _, ospo = oracle.estimate_pairs(g, 5, 0.5, 5, per_owner=True)
     assert s == os_ and np.array_equal(spo, ospo)
+
+
+@pytest.mark.parametrize("n,p,k", [(520, 0.5, 5), (560, 0.75, 5), (420, 0.9, 5), (700, 0.4, 6), (440, 0.62, 6)])
+def test_closed_or_searched_by_density(kc, n, p, k):
+    """Owners of 8 and 16 words of a dense graph, and of the same graph among 20,000 vertices without edges: whether
+    their sets are closed or searched depends on the density of the whole."""
+    g = kcgen.random_small(n, p, 5)
+    G = kc.orient(g.off, g.adj)
+    assert 128 < G.max_dplus <= 512
+    off = np.concatenate([g.off, np.full(20000 - n, g.off[-1])])
+    H = kc.orient(off, g.adj)
+    t, pv, po = kc.count(G, k, per_vertex=True, per_owner=True)
+    tt, ppv, ppo = kc.count(H, k, per_vertex=True, per_owner=True)
+    assert t == tt and np.array_equal(pv, ppv[:n]) and np.array_equal(po, ppo[:n])
+    for X in (G, H):
+        x, _, xo = kc.count(X, k, per_owner=True)
+        assert x == t and np.array_equal(xo[:n], po) and kc.count_batch([X, X], k) == [t, t]
+    for c in (2, 5):
+        a, b = kc.estimate(G, k, c, 3, per_owner=True), kc.estimate(H, k, c, 3, per_owner=True)
+        assert a[0] == b[0] and np.array_equal(a[2], b[2][:n])
+    for q in (0.5, 0.7, 0.85, 0.95):
+        a, b = kc.estimate_pairs(G, k, q, 3, per_owner=True), kc.estimate_pairs(H, k, q, 3, per_owner=True)
+        assert a[0] == b[0] and np.array_equal(a[2], b[2][:n])
+
+
+@pytest.mark.parametrize("ps", [(0.5, 0.6), (0.5, 0.95), (0.02, 0.6), (0.3,)])
+def test_batches_by_density(kc, ps):
+    # 16-word owners in graphs of middling density, in one denser, beside a sparse graph, and none at all
+    graphs = [kcgen.random_small(560, p, 7) for p in ps]
+    Gs = [kc.orient(g.off, g.adj) for g in graphs]
+    for k in (5, 6):
+        assert kc.count_batch(Gs, k) == [kc.count(G, k, per_vertex=True)[0] for G in Gs]
