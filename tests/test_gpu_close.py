@@ -1,9 +1,8 @@
 """Candidate sets closed on a compact copy of their subgraph (csrc/close.cu):
 every row width of the copy (1..16 words), both sides of the flip to the
 complement, against the oracle where it can enumerate the cliques, against
-closed forms, and against the ordered search (KC_PARAM_COMPLEMENT = 0).
-
-Sets are closed at k = 5 and 6; the cases at k = 7 run the ordered search over the same graphs."""
+closed forms, and against the ordered search (KC_PARAM_COMPLEMENT = 0)."""
+# Sets are closed at k = 5 and 6; the cases at k = 7 run the ordered search over the same graphs.
 from math import comb
 
 import numpy as np
